@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS) adjoint_kernel(AdjointLaunch A
                 float f[3], delta;
                 place(rp, step, L.grid.n, j, ip, f, delta);
                 if (ESL && (dist[brick_of(L.bricks, ip)] != 0 ||
-                            (L.cells && !cell_open(L.cells, L.cwx, L.grid.n, ip))))
+                            (L.cells && !cell_open(L.cells, L.grid.n, ip))))
                     continue;
                 SampleEval e;
                 eval_sample(L, ip, f, delta, e);

@@ -273,11 +273,9 @@ cudaError_t launch_occupancy(const void *mn, const void *mx, int dtype, long nbr
 // Cell c (per axis c = -1 .. n-1, index c' = c + 1) holds the samples with floor(p) = c; their
 // 64 cubic taps are voxels c-1 .. c+2, i.e. padded indices c' .. c'+3. The B-spline weights are
 // non-negative and sum to one, so such a sample lies in [min, max] of the taps (up to float
-// rounding, which the +-1 index margin covers). Bit c' of the mask is the occupancy rule on
-// that range: open when an entry of non-zero opacity lies in
-// [floor(u(min)) - 1, ceil(u(max)) + 1]; a sample in a clear cell has opacity exactly zero.
-// Bits: words of 32 cells along x, word (c'_z * (ny + 1) + c'_y) * cwx + c'_x / 32, bit
-// c'_x % 32.
+// rounding, which the +-1 index margin covers). A cell is open when an entry of non-zero
+// opacity lies in [floor(u(min)) - 1, ceil(u(max)) + 1] (the occupancy rule); a sample in a
+// clear cell has opacity exactly zero. Layout of the mask: cell_open (vrc_internal.h).
 //
 // The rule is evaluated without a min/max: u is monotone in the value, so the range is the
 // union of the taps' own index intervals [floor(u_i) - 1, ceil(u_i) + 1], and it holds no
@@ -286,166 +284,232 @@ cudaError_t launch_occupancy(const void *mn, const void *mx, int dtype, long nbr
 // when none does), and a cell is clear exactly when its 64 bytes are equal and non-zero,
 // i.e. when their bitwise OR equals their bitwise AND and is non-zero.
 //
-// Pass 1 (zero_run_id_kernel) writes that byte for every padded voxel, 8 voxels per thread.
-// Pass 2 (cellmask_kernel) gives each thread 4 cells along x (one 32-bit word of bytes and the
-// next) in one (y, z-run) column: per padded z slice it ORs / ANDs the 4 rows of the y window
-// into a register ring of the last 4 slices, then the z window over the ring, then the x
-// window by funnel shifts; 8 lanes combine their 4 bits into one mask word.
-constexpr int CM_ZC = 16;  // cells per thread along z
+// Only cells of occupied bricks are worked out: a brick's [min, max] covers the taps of all its
+// cells (the apron), so the cells of an empty brick are clear, by the same rule. The unit of
+// work is a tile of 8^3 cells, 8t - 8 .. 8t - 1 per axis, which lies in one brick (tile 0 holds
+// the cells -1). A warp takes 4 tiles in a row along x, writes zeros for those whose brick is
+// empty, and works through the others one by one: the tile's 11 x 11 rows of 11 voxels are read
+// with vector loads (8t - 8 is a 16-byte boundary of the padded row), reduced to run ids and
+// ORed / ANDed along x in registers, the y and z windows are taken from shared memory, and the
+// bits of a 4^3 block are gathered by a warp reduction.
+// Bound: latency and issue of the occupied tiles (about 15 ALU operations a voxel). 512^2 x 400
+// int16 with bone and vessels visible: 43 us, against 240 us for two passes over the
+// whole volume (run ids of every voxel to memory, then every cell's windows).
+constexpr int CM_TILES = 4, CM_WARPS = 4;  // tiles a warp, warps a CTA
+constexpr int CM_W = 11;  // voxels per axis that the cells of a tile read
 
-template <typename T>
-__device__ __forceinline__ void load8(const T *__restrict__ src, long g, float v[8]) {
-    const uint4 q = __ldg((const uint4 *)src + g);  // 8 two-byte values
-    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        v[2 * e] = (float)(T)(w[e] & 0xffffu);
-        v[2 * e + 1] = (float)(T)(w[e] >> 16);
+// Table of the run id of a voxel's index interval: entry f for u = f exactly, entry 256 + f for
+// u in (f, f + 1); zero when no single zero run holds the interval.
+__device__ __forceinline__ void zero_run_table(const uint8_t *__restrict__ zrun, uint8_t *tab,
+                                               int nthreads) {
+    for (int i = threadIdx.x; i < 512; i += nthreads) {
+        const int f = i & 255;
+        const int k0 = max(f - 1, 0), k1 = min(f + 1 + (i >> 8), 255);
+        tab[i] = zrun[k0] == zrun[k1] ? zrun[k0] : (uint8_t)0;
     }
 }
 
-template <>
-__device__ __forceinline__ void load8<float>(const float *__restrict__ src, long g, float v[8]) {
-    const float4 a = __ldg((const float4 *)src + 2 * g), b = __ldg((const float4 *)src + 2 * g + 1);
-    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
-    v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+__device__ __forceinline__ uint32_t zero_run_of(const uint8_t *tab, float v, float lo, float du) {
+    const float u = u_index(v, lo, du);
+    int f;
+    const float fl = floor_small(u, f);
+    return tab[f + (u > fl ? 256 : 0)];
+}
+
+// The run ids of padded elements x0 + 1 .. x0 + 11 of a row (x0 a multiple of 8), as bytes of
+// w[0 .. 2]; elements outside the row (x0 = -8, and past its end) are read by no cell.
+template <typename T>
+__device__ __forceinline__ void run_id_row(const T *__restrict__ row, int x0, int pnx,
+                                           const uint8_t *tab, float lo, float du,
+                                           uint32_t w[3]) {
+    T v[12] = {};
+    if constexpr (sizeof(T) == 2) {
+        if (x0 >= 0) {
+            const uint4 a = __ldg((const uint4 *)(row + x0));
+            memcpy(v, &a, 16);
+        }
+        if (x0 + 8 < pnx) {
+            const uint2 b = __ldg((const uint2 *)(row + x0 + 8));
+            memcpy(v + 8, &b, 8);
+        }
+    } else {
+        if (x0 >= 0) {
+            const float4 a = __ldg((const float4 *)(row + x0));
+            const float4 b = __ldg((const float4 *)(row + x0) + 1);
+            memcpy(v, &a, 16);
+            memcpy(v + 4, &b, 16);
+        }
+        if (x0 + 8 < pnx) {
+            const float4 c = __ldg((const float4 *)(row + x0 + 8));
+            memcpy(v + 8, &c, 16);
+        }
+    }
+    w[0] = w[1] = w[2] = 0u;
+#pragma unroll
+    for (int e = 0; e < CM_W; ++e)
+        w[e >> 2] |= zero_run_of(tab, (float)v[e + 1], lo, du) << (8 * (e & 3));
+}
+
+// Bits of the bytes i of (o, a) whose cell is open: o != a or o == 0.
+__device__ __forceinline__ uint32_t open_nibble(uint32_t o, uint32_t a) {
+    auto nz = [](uint32_t v) { return (((v & 0x7f7f7f7fu) + 0x7f7f7f7fu) | v) & 0x80808080u; };
+    const uint32_t m = (nz(o ^ a) | (nz(o) ^ 0x80808080u)) >> 7;
+    return (m | (m >> 7) | (m >> 14) | (m >> 21)) & 0xfu;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) zero_run_id_kernel(const T *__restrict__ src, long n8,
-                                                          const uint8_t *__restrict__ zrun,
-                                                          float lo, float du,
-                                                          uint2 *__restrict__ out) {
-    __shared__ uint8_t rid[256];
-    rid[threadIdx.x] = zrun[threadIdx.x];
+__global__ void __launch_bounds__(32 * CM_WARPS)
+    cellmask_kernel(VolView v, const uint8_t *__restrict__ occ, int shift, int nbx, int nby,
+                    const uint8_t *__restrict__ zrun, float lo, float du,
+                    uint32_t *__restrict__ cells) {
+    __shared__ uint8_t tab[512];
+    __shared__ uint4 s_rows[CM_WARPS][CM_W * CM_W];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint4 *rows = s_rows[warp];
+    const int nfx = cell_blocks(v.n[0]), nfy = cell_blocks(v.n[1]), nfz = cell_blocks(v.n[2]);
+    const int ntx = cell_tiles(v.n[0]), nty = cell_tiles(v.n[1]), ntz = cell_tiles(v.n[2]);
+    const unsigned gx = (unsigned)(ntx + CM_TILES - 1) / CM_TILES;
+    const unsigned unit = blockIdx.x * CM_WARPS + warp;
+    const int t0 = (int)(unit % gx) * CM_TILES;
+    const int ty = (int)((unit / gx) % nty), tz = (int)(unit / (gx * nty));
+
+    // the tiles with an occupied brick; zeros for the others (lane: row of blocks, tile)
+    unsigned met = 0;
+    if (tz < ntz) {
+        const int tile = lane & 3, tx = t0 + tile;
+        const int to_brick = shift - 3;
+        bool any = false;
+        if (tx < ntx)
+            any = occ[((long)(max(tz - 1, 0) >> to_brick) * nby + (max(ty - 1, 0) >> to_brick)) *
+                          nbx + (max(tx - 1, 0) >> to_brick)] != 0;
+        met = __ballot_sync(0xffffffffu, any) & ((1u << CM_TILES) - 1u);
+        const int by = 2 * ty - 1 + ((lane >> 2) & 1), bz = 2 * tz - 1 + ((lane >> 3) & 1);
+        if (lane < 16 && tx < ntx && !any && (unsigned)by < (unsigned)nfy &&
+            (unsigned)bz < (unsigned)nfz) {
+            uint2 *o = (uint2 *)cells + ((long)bz * nfy + by) * nfx + 2 * tx;
+            if (tx > 0) o[-1] = make_uint2(0u, 0u);
+            if (2 * tx < nfx) o[0] = make_uint2(0u, 0u);
+        }
+    }
+    if (!__syncthreads_or(met != 0)) return;
+    zero_run_table(zrun, tab, 32 * CM_WARPS);
     __syncthreads();
-    for (long g = blockIdx.x * 256L + threadIdx.x; g < n8; g += (long)gridDim.x * 256) {
-        float v[8];
-        load8<T>(src, g, v);
-        uint32_t w[2] = {0u, 0u};
+    const T *base = (const T *)v.base;
+    for (; met; met &= met - 1) {
+        const int tx = t0 + __ffs(met) - 1;
+        __syncwarp();  // the rows of the tile before have been read
+        for (int r = lane; r < CM_W * CM_W; r += 32) {
+            const int y = min(max(8 * ty - 7 + r % CM_W, 0), v.pny - 1);
+            const int z = min(max(8 * tz - 7 + r / CM_W, 0), v.pnz - 1);
+            uint32_t w[3];
+            run_id_row<T>(base + ((long)z * v.pny + y) * v.pnx, 8 * tx - 8, v.pnx, tab, lo, du, w);
+            // byte i of o / a: OR / AND over the columns i .. i+3 of cell i
+            uint32_t o[2], a[2];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const float u = u_index(v[e], lo, du);
-            const int k0 = max((int)floorf(u) - 1, 0);
-            const int k1 = min((int)ceilf(u) + 1, 255);
-            const uint32_t r0 = rid[k0], r1 = rid[k1];
-            w[e >> 2] |= (r0 == r1 ? r0 : 0u) << (8 * (e & 3));
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t w1 = __funnelshift_r(w[h], w[h + 1], 8);
+                const uint32_t w2 = __funnelshift_r(w[h], w[h + 1], 16);
+                const uint32_t w3 = __funnelshift_r(w[h], w[h + 1], 24);
+                o[h] = (w[h] | w1) | (w2 | w3);
+                a[h] = (w[h] & w1) & (w2 & w3);
+            }
+            rows[r] = make_uint4(o[0], o[1], a[0], a[1]);
         }
-        out[g] = make_uint2(w[0], w[1]);
-    }
-}
-
-// gid: the run-id bytes as words (wpr words per padded row); kpad: threads per (y, z-run)
-// column, a multiple of 8 >= ceil((nx + 1) / 4), so that the 8 lanes building one mask word
-// share a column.
-__global__ void __launch_bounds__(128) cellmask_kernel(const uint32_t *__restrict__ gid, int wpr,
-                                                       int pny, int nx, int ny, int nz,
-                                                       uint32_t *__restrict__ cells, int cwx,
-                                                       int kpad) {
-    const long t = blockIdx.x * 128L + threadIdx.x;
-    const int lane = threadIdx.x & 31;
-    const int k = (int)(t % kpad);  // cells 4k .. 4k+3 (k & 7 == lane & 7)
-    const long col = t / kpad;      // the same for the 8 lanes of a mask word
-    const int cy = (int)(col % (ny + 1));
-    const int cz0 = (int)(col / (ny + 1)) * CM_ZC;
-    if (cz0 > nz) return;  // past the last column: whole groups of 8 lanes leave
-    const int cz1 = min(cz0 + CM_ZC, nz + 1);
-    const bool kval = k < (nx + 1 + 3) / 4;
-    // cells past nx read clamped words; their bits are never used
-    const int kw0 = min(k, wpr - 1), kw1 = min(k + 1, wpr - 1);
-    uint32_t ro0[4] = {0u, 0u, 0u, 0u}, ra0[4] = {0u, 0u, 0u, 0u};  // newest first
-    uint32_t ro1[4] = {0u, 0u, 0u, 0u}, ra1[4] = {0u, 0u, 0u, 0u};
-    // padded slice zp holds taps of cells zp - 3 .. zp; rows cy .. cy+3 the y window. The
-    // words of slice zp + 1 are loaded while slice zp is reduced.
-    uint32_t nw0[4], nw1[4];
-    {
-        const uint32_t *row = gid + ((long)cz0 * pny + cy) * wpr;
+        __syncwarp();
+        const int y = lane & 7, cy = 8 * ty - 8 + y;
+        const int cx = 8 * tx - 8;
+        // cells of the tile inside the volume, -1 .. n-1, as bits
+        const unsigned inx = (tx == 0 ? 0x80u : 0xffu) & ((2u << min(v.n[0] - 1 - cx, 7)) - 1u);
 #pragma unroll
-        for (int dy = 0; dy < 4; ++dy) {
-            nw0[dy] = __ldg(row + dy * wpr + kw0);
-            nw1[dy] = __ldg(row + dy * wpr + kw1);
-        }
-    }
-    for (int zp = cz0; zp < cz1 + 3; ++zp) {
-        uint32_t o0 = 0u, a0 = 0xffffffffu, o1 = 0u, a1 = 0xffffffffu;
+        for (int h = 0; h < 2; ++h) {  // cells of the lower, then the upper 4^3 blocks in z
+            const int z = 4 * h + (lane >> 3), cz = 8 * tz - 8 + z;
+            uint32_t o0 = 0u, o1 = 0u, a0 = 0xffffffffu, a1 = 0xffffffffu;
 #pragma unroll
-        for (int dy = 0; dy < 4; ++dy) {
-            o0 |= nw0[dy];
-            a0 &= nw0[dy];
-            o1 |= nw1[dy];
-            a1 &= nw1[dy];
-        }
-        if (zp + 1 < cz1 + 3) {
-            const uint32_t *row = gid + ((long)(zp + 1) * pny + cy) * wpr;
+            for (int dz = 0; dz < 4; ++dz) {
 #pragma unroll
-            for (int dy = 0; dy < 4; ++dy) {
-                nw0[dy] = __ldg(row + dy * wpr + kw0);
-                nw1[dy] = __ldg(row + dy * wpr + kw1);
+                for (int dy = 0; dy < 4; ++dy) {
+                    const uint4 q = rows[(z + dz) * CM_W + y + dy];
+                    o0 |= q.x;
+                    o1 |= q.y;
+                    a0 &= q.z;
+                    a1 &= q.w;
+                }
+            }
+            const bool yz = cy >= -1 && cy < v.n[1] && cz >= -1 && cz < v.n[2];
+            const uint32_t n0 = yz ? open_nibble(o0, a0) & inx : 0u;
+            const uint32_t n1 = yz ? open_nibble(o1, a1) & (inx >> 4) : 0u;
+            // one 32-bit half block per 8 lanes: 4 rows y x 2 slices z
+            const unsigned mask = 0x0f0fu << (4 * ((lane >> 2) & 1) + 16 * (lane >> 4));
+            const int sh = 16 * ((lane >> 3) & 1) + 4 * (lane & 3);
+            const uint32_t w0 = __reduce_or_sync(mask, n0 << sh);
+            const uint32_t w1 = __reduce_or_sync(mask, n1 << sh);
+            const int by = 2 * ty - 1 + ((lane >> 2) & 1), bz = 2 * tz - 1 + h;
+            if ((lane & 11) == 0 && (unsigned)by < (unsigned)nfy && (unsigned)bz < (unsigned)nfz) {
+                uint32_t *out = cells + 2 * (((long)bz * nfy + by) * nfx + 2 * tx) + (lane >> 4);
+                if (tx > 0) out[-2] = w0;
+                if (2 * tx < nfx) out[0] = w1;
             }
         }
-#pragma unroll
-        for (int r = 3; r > 0; --r) {
-            ro0[r] = ro0[r - 1];
-            ra0[r] = ra0[r - 1];
-            ro1[r] = ro1[r - 1];
-            ra1[r] = ra1[r - 1];
-        }
-        ro0[0] = o0;
-        ra0[0] = a0;
-        ro1[0] = o1;
-        ra1[0] = a1;
-        if (zp < cz0 + 3) continue;
-        const uint32_t O0 = (ro0[0] | ro0[1]) | (ro0[2] | ro0[3]);
-        const uint32_t A0 = (ra0[0] & ra0[1]) & (ra0[2] & ra0[3]);
-        const uint32_t O1 = (ro1[0] | ro1[1]) | (ro1[2] | ro1[3]);
-        const uint32_t A1 = (ra1[0] & ra1[1]) & (ra1[2] & ra1[3]);
-        // byte i of Ox / Ax: OR / AND over the columns 4k+i .. 4k+i+3 of cell 4k+i
-        const uint32_t Ox = O0 | __funnelshift_r(O0, O1, 8) | __funnelshift_r(O0, O1, 16) |
-                            __funnelshift_r(O0, O1, 24);
-        const uint32_t Ax = A0 & __funnelshift_r(A0, A1, 8) & __funnelshift_r(A0, A1, 16) &
-                            __funnelshift_r(A0, A1, 24);
-        uint32_t open = 0u;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint32_t ob = (Ox >> (8 * i)) & 0xffu, ab = (Ax >> (8 * i)) & 0xffu;
-            open |= (uint32_t)(!(ob == ab && ob != 0u)) << i;
-        }
-        if (!kval) open = 0u;
-        const uint32_t w = __reduce_or_sync(0xffu << (lane & 24), open << (4 * (k & 7)));
-        if ((lane & 7) == 0 && (k >> 3) < cwx)
-            cells[((long)(zp - 3) * (ny + 1) + cy) * cwx + (k >> 3)] = w;
     }
 }
 
-long cellmask_words(const int n[3]) {
+size_t cellmask_bytes(const int n[3]) {
+    return 8 * (size_t)cell_blocks(n[0]) * cell_blocks(n[1]) * cell_blocks(n[2]);
+}
+
+cudaError_t launch_cellmask(const VolView &v, int B, const int nb[3], const uint8_t *occ,
+                            const uint8_t *zrun_dev, float lo, float du, uint32_t *cells,
+                            cudaStream_t st) {
+    const long units = (long)((cell_tiles(v.n[0]) + CM_TILES - 1) / CM_TILES) *
+                       cell_tiles(v.n[1]) * cell_tiles(v.n[2]);
+    const unsigned blocks = (unsigned)((units + CM_WARPS - 1) / CM_WARPS);
+    const int shift = B == 16 ? 4 : 3;
+    switch (v.dtype) {
+    case DT_U16:
+        cellmask_kernel<uint16_t><<<blocks, 32 * CM_WARPS, 0, st>>>(v, occ, shift, nb[0], nb[1],
+                                                                    zrun_dev, lo, du, cells);
+        break;
+    case DT_I16:
+        cellmask_kernel<int16_t><<<blocks, 32 * CM_WARPS, 0, st>>>(v, occ, shift, nb[0], nb[1],
+                                                                   zrun_dev, lo, du, cells);
+        break;
+    default:
+        cellmask_kernel<float><<<blocks, 32 * CM_WARPS, 0, st>>>(v, occ, shift, nb[0], nb[1],
+                                                                 zrun_dev, lo, du, cells);
+    }
+    return cudaGetLastError();
+}
+
+// The mask as rows of 32 cells along x (vrc_cellmask_get): word (c'_z (ny + 1) + c'_y) cwx +
+// c'_x / 32, bit c'_x % 32, c' = c + 1. One thread per word.
+__global__ void cellmask_rows_kernel(const uint32_t *__restrict__ cells, int nx, int ny, int nz,
+                                     int cwx, uint32_t *__restrict__ out) {
+    const long total = (long)cwx * (ny + 1) * (nz + 1);
+    const int nfx = cell_blocks(nx), nfy = cell_blocks(ny);
+    for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total;
+         i += (long)gridDim.x * blockDim.x) {
+        const int wx = (int)(i % cwx), y = (int)((i / cwx) % (ny + 1)) + 3;
+        const int z = (int)(i / ((long)cwx * (ny + 1))) + 3;
+        // cells c' = 32 wx .. + 31 are bits 3 .. 34 of the 9 nibbles from block 8 wx
+        const uint32_t *row = cells + 2 * (((long)(z >> 2) * nfy + (y >> 2)) * nfx) + ((z >> 1) & 1);
+        unsigned long long w = 0ull;
+        for (int k = 0; k < 9 && 8 * wx + k < nfx; ++k)
+            w |= (unsigned long long)((row[2 * (8 * wx + k)] >> (16 * (z & 1) + 4 * (y & 3))) & 0xfu)
+                 << (4 * k);
+        out[i] = (uint32_t)(w >> 3);
+    }
+}
+
+long cellmask_row_words(const int n[3]) {
     return (long)((n[0] + 1 + 31) / 32) * (n[1] + 1) * (n[2] + 1);
 }
 
-size_t cellmask_scratch_bytes(const VolView &v) { return (size_t)v.pnx * v.pny * v.pnz; }
-
-cudaError_t launch_cellmask(const VolView &v, const uint8_t *zrun_dev, float lo, float du,
-                            uint8_t *scratch, uint32_t *cells, cudaStream_t st) {
-    const long n8 = (long)v.pnx * v.pny * v.pnz / 8;  // pnx is a multiple of 8
-    long b1 = (n8 + 255) / 256;
-    if (b1 > 152L * 16) b1 = 152L * 16;
-    switch (v.dtype) {
-    case DT_U16:
-        zero_run_id_kernel<uint16_t><<<(unsigned)b1, 256, 0, st>>>(
-            (const uint16_t *)v.base, n8, zrun_dev, lo, du, (uint2 *)scratch);
-        break;
-    case DT_I16:
-        zero_run_id_kernel<int16_t><<<(unsigned)b1, 256, 0, st>>>(
-            (const int16_t *)v.base, n8, zrun_dev, lo, du, (uint2 *)scratch);
-        break;
-    default:
-        zero_run_id_kernel<float><<<(unsigned)b1, 256, 0, st>>>(
-            (const float *)v.base, n8, zrun_dev, lo, du, (uint2 *)scratch);
-    }
-    const int cwx = (v.n[0] + 1 + 31) / 32;
-    const int kpad = ((v.n[0] + 1 + 3) / 4 + 7) / 8 * 8;
-    const long threads = (long)kpad * (v.n[1] + 1) * ((v.n[2] + 1 + CM_ZC - 1) / CM_ZC);
-    cellmask_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(
-        (const uint32_t *)scratch, v.pnx / 4, v.pny, v.n[0], v.n[1], v.n[2], cells, cwx, kpad);
+cudaError_t launch_cellmask_rows(const uint32_t *cells, const int n[3], uint32_t *out,
+                                 cudaStream_t st) {
+    const long words = cellmask_row_words(n);
+    const long blocks = (words + 255) / 256;
+    cellmask_rows_kernel<<<(unsigned)(blocks > 152L * 32 ? 152L * 32 : blocks), 256, 0, st>>>(
+        cells, n[0], n[1], n[2], (n[0] + 1 + 31) / 32, out);
     return cudaGetLastError();
 }
 
@@ -490,82 +554,72 @@ cudaError_t launch_preint_table(const float4 *rgba, float ds, float4 *tab, cudaS
 // dist[oct][b] = 0 for an occupied brick, else the smallest r >= 1 such that the forward box
 // of bricks {b + t : t_k between 0 and r s_k} holds an occupied brick (capped at 255). Every
 // brick of the forward box of extent r - 1 is empty, so a ray whose direction lies in that
-// octant may leap from b to the exit of that box. Computed from a summed-volume table of the
-// occupancy bytes; octant index = (sx < 0) | (sy < 0) << 1 | (sz < 0) << 2.
+// octant may leap from b to the exit of that box. Octant index = (sx < 0) | (sy < 0) << 1 |
+// (sz < 0) << 2.
+//
+// That is the distance to the nearest occupied brick ahead in the maximum norm, which separates
+// by axis: with g the distances along x alone, f(y) = min over d >= 0 of max(d, g(y + d sy)),
+// and the same again along z. Pass x finds the next set bit of the row's occupancy bits (2
+// fields), passes y and z search forward until d reaches the best value (4, then 8 fields); a
+// step reads consecutive bytes across a warp. Latency-bound (a field of 64 x 64 x 50 bricks is
+// 0.2 MB): 31 us for the three passes, against 108 us for a summed-volume table by serial
+// prefix sums and a binary search per brick and octant.
+constexpr int DX_WARPS = 4;
 
-// S has (nbz+1) x (nby+1) x (nbx+1) ints; first pass: S[z+1][y+1][x+1] = sum_{x'<=x} occ.
-__global__ void svt_x_kernel(const uint8_t *__restrict__ occ, int nbx, int nby, int nbz,
-                             int *__restrict__ S) {
-    const int sx = nbx + 1, sy = nby + 1;
-    long lines = (long)(nby + 1) * (nbz + 1);
-    for (long l = blockIdx.x * (long)blockDim.x + threadIdx.x; l < lines;
-         l += (long)gridDim.x * blockDim.x) {
-        int y = (int)(l % sy), z = (int)(l / sy);
-        int *row = S + ((long)z * sy + y) * sx;
-        int acc = 0;
-        row[0] = 0;
-        for (int x = 0; x < nbx; ++x) {
-            if (y > 0 && z > 0) acc += occ[((long)(z - 1) * nby + (y - 1)) * nbx + x];
-            row[x + 1] = acc;
-        }
+// One warp per row (y, z) of bricks, 32 at a time, once in each direction.
+__global__ void __launch_bounds__(32 * DX_WARPS) dist_x_kernel(const uint8_t *__restrict__ occ,
+                                                               int nbx, long rows,
+                                                               uint8_t *__restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    const long row = (long)blockIdx.x * DX_WARPS + (threadIdx.x >> 5);
+    if (row >= rows) return;
+    const uint8_t *o = occ + row * nbx;
+    uint8_t *fwd = out + row * nbx, *bwd = fwd + rows * nbx;
+    // carry: distance from the last brick handled to the nearest occupied one at or before it
+    int carry = 255;
+    for (int x0 = 0; x0 < nbx; x0 += 32) {
+        const int x = x0 + lane;
+        const unsigned bits = __ballot_sync(0xffffffffu, x < nbx && o[x] != 0);
+        const unsigned at = bits & (0xffffffffu >> (31 - lane));  // bricks x0 .. x
+        const int d = at ? lane - (31 - __clz(at)) : min(carry + lane + 1, 255);
+        if (x < nbx) bwd[x] = (uint8_t)d;
+        carry = __shfl_sync(0xffffffffu, d, 31);
+    }
+    carry = 255;
+    for (int x0 = (nbx - 1) & ~31; x0 >= 0; x0 -= 32) {
+        const int x = x0 + lane;
+        const unsigned bits = __ballot_sync(0xffffffffu, x < nbx && o[x] != 0);
+        const unsigned at = bits & (0xffffffffu << lane);  // bricks x .. x0 + 31
+        // past the row's end there is nothing: a full carry
+        const int d = at ? __ffs(at) - 1 - lane : min(carry + 32 - lane, 255);
+        if (x < nbx) fwd[x] = (uint8_t)d;
+        carry = __shfl_sync(0xffffffffu, d, 0);
     }
 }
 
-// prefix sums along y (axis = 1) or z (axis = 2) of S in place
-__global__ void svt_yz_kernel(int nbx, int nby, int nbz, int axis, int *__restrict__ S) {
-    const long sx = nbx + 1, sy = nby + 1, sz = nbz + 1;
-    const long lines = axis == 1 ? sx * sz : sx * sy;
-    const long stride = axis == 1 ? sx : sx * sy;
-    const int len = axis == 1 ? (int)sy : (int)sz;
-    for (long l = blockIdx.x * (long)blockDim.x + threadIdx.x; l < lines;
-         l += (long)gridDim.x * blockDim.x) {
-        long base = axis == 1 ? (l % sx) + (l / sx) * sx * sy : l;
-        int acc = 0;
-        for (int i = 0; i < len; ++i) {
-            acc += S[base + i * stride];
-            S[base + i * stride] = acc;
+// Pass along an axis of `len` bricks spaced `stride` apart, one field per blockIdx.y: fields NIN
+// in, 2 NIN out, field f + NIN h from field f searching towards +(h = 0) or -(h = 1).
+template <int NIN>
+__global__ void __launch_bounds__(256) dist_axis_kernel(const uint8_t *__restrict__ in, unsigned n,
+                                                        unsigned len, unsigned stride,
+                                                        uint8_t *__restrict__ out) {
+    const int h = blockIdx.y / NIN;
+    const uint8_t *f = in + (size_t)(blockIdx.y % NIN) * n;
+    uint8_t *o = out + (size_t)blockIdx.y * n;
+    const int s = h ? -(int)stride : (int)stride;
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n; i += gridDim.x * 256u) {
+        const uint8_t *p = f + i;
+        const int pos = (int)((i / stride) % len);
+        const int room = h ? pos : (int)len - 1 - pos;  // bricks ahead
+        int best = p[0];
+        for (int d = 1; d < best && d <= room; d += 4) {
+            int g[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) g[k] = p[(long)min(d + k, room) * s];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) best = min(best, max(d + k, g[k]));
         }
-    }
-}
-
-__device__ __forceinline__ int svt_at(const int *S, int sx, int sy, int x, int y, int z) {
-    return S[((long)z * sy + y) * sx + x];
-}
-
-__global__ void box_dist_kernel(const uint8_t *__restrict__ occ, const int *__restrict__ S,
-                                int nbx, int nby, int nbz, uint8_t *__restrict__ dist) {
-    const int sx = nbx + 1, sy = nby + 1;
-    const long n = (long)nbx * nby * nbz;
-    for (long q = blockIdx.x * (long)blockDim.x + threadIdx.x; q < 8 * n;
-         q += (long)gridDim.x * blockDim.x) {
-        const int oct = (int)(q / n);
-        const long i = q % n;
-        if (occ[i]) {
-            dist[q] = 0;
-            continue;
-        }
-        const int bx = (int)(i % nbx), by = (int)((i / nbx) % nby), bz = (int)(i / ((long)nbx * nby));
-        const bool nx_ = oct & 1, ny_ = oct & 2, nz_ = oct & 4;
-        auto count = [&](int r) {
-            int x0 = nx_ ? max(bx - r, 0) : bx, x1 = (nx_ ? bx : min(bx + r, nbx - 1)) + 1;
-            int y0 = ny_ ? max(by - r, 0) : by, y1 = (ny_ ? by : min(by + r, nby - 1)) + 1;
-            int z0 = nz_ ? max(bz - r, 0) : bz, z1 = (nz_ ? bz : min(bz + r, nbz - 1)) + 1;
-            return svt_at(S, sx, sy, x1, y1, z1) - svt_at(S, sx, sy, x0, y1, z1) -
-                   svt_at(S, sx, sy, x1, y0, z1) - svt_at(S, sx, sy, x1, y1, z0) +
-                   svt_at(S, sx, sy, x0, y0, z1) + svt_at(S, sx, sy, x0, y1, z0) +
-                   svt_at(S, sx, sy, x1, y0, z0) - svt_at(S, sx, sy, x0, y0, z0);
-        };
-        int lo = 1, hi = 255;  // smallest r in [lo, hi] with count(r) > 0, else 255
-        if (count(hi) == 0) {
-            dist[q] = 255;
-            continue;
-        }
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (count(mid) > 0) hi = mid;
-            else lo = mid + 1;
-        }
-        dist[q] = (uint8_t)lo;
+        o[i] = (uint8_t)best;
     }
 }
 
@@ -573,21 +627,18 @@ size_t box_dist_scratch_bytes(const int nb[3]) {
     return (size_t)(nb[0] + 1) * (nb[1] + 1) * (nb[2] + 1) * sizeof(int);
 }
 
+// The x fields go through the first quarter of `dist`, the y fields (4 bytes a brick) through
+// `scratch`.
 cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], int *scratch, uint8_t *dist,
                              cudaStream_t st) {
-    const int threads = 256;
-    auto grid_for = [&](long n) {
-        long b = (n + threads - 1) / threads;
-        return (unsigned)(b < 1 ? 1 : (b > 152L * 16 ? 152L * 16 : b));
-    };
-    svt_x_kernel<<<grid_for((long)(nb[1] + 1) * (nb[2] + 1)), threads, 0, st>>>(occ, nb[0], nb[1],
-                                                                                 nb[2], scratch);
-    svt_yz_kernel<<<grid_for((long)(nb[0] + 1) * (nb[2] + 1)), threads, 0, st>>>(nb[0], nb[1],
-                                                                                  nb[2], 1, scratch);
-    svt_yz_kernel<<<grid_for((long)(nb[0] + 1) * (nb[1] + 1)), threads, 0, st>>>(nb[0], nb[1],
-                                                                                  nb[2], 2, scratch);
-    box_dist_kernel<<<grid_for(8L * nb[0] * nb[1] * nb[2]), threads, 0, st>>>(
-        occ, scratch, nb[0], nb[1], nb[2], dist);
+    const long n = (long)nb[0] * nb[1] * nb[2], rows = (long)nb[1] * nb[2];
+    const unsigned blocks = (unsigned)((n + 255) / 256 > 152L * 64 ? 152L * 64 : (n + 255) / 256);
+    uint8_t *yf = (uint8_t *)scratch;
+    dist_x_kernel<<<(unsigned)((rows + DX_WARPS - 1) / DX_WARPS), 32 * DX_WARPS, 0, st>>>(
+        occ, nb[0], rows, dist);
+    dist_axis_kernel<2><<<dim3(blocks, 4), 256, 0, st>>>(dist, (unsigned)n, nb[1], nb[0], yf);
+    dist_axis_kernel<4><<<dim3(blocks, 8), 256, 0, st>>>(yf, (unsigned)n, nb[2], nb[0] * nb[1],
+                                                         dist);
     return cudaGetLastError();
 }
 

@@ -86,7 +86,7 @@ __device__ __forceinline__ void group_march(const RenderLaunch &L, const RayPos 
                     cache_occ = dist[lin] == 0;
                 }
                 in_occ = cache_occ;
-                live = in_occ && (!L.cells || cell_open(L.cells, L.cwx, L.grid.n, ip));
+                live = in_occ && (!L.cells || cell_open(L.cells, L.grid.n, ip));
             }
             if (live) {
                 const float4 rgba = sample_rgba<MODE>(L.rep, L.tf, ip, f, df, &L.phong);

@@ -21,11 +21,11 @@ namespace vrc {
 
 namespace {
 
-// One warp per brick. Cell c (per axis -1 .. n-1) sits at mask index c + 1; brick b holds the
+// One warp per brick. Cells run from -1 to n-1 per axis; brick b holds the
 // cells [bB, bB + B) cut to n - 1, brick 0 also the cell -1. Each lane takes whole rows (y, z)
-// of the brick's cells and extracts their x bits (at most B + 1 bits, two words at most).
+// of the brick's cells and gathers their x bits (at most B + 1, 4 per block of the mask).
 __global__ void __launch_bounds__(256) brick_aabb_kernel(const uint32_t *__restrict__ cells,
-                                                         int cwx, int nx, int ny, int nz,
+                                                         int nx, int ny, int nz,
                                                          int B, int nbx, int nby, int nbz,
                                                          const uint8_t *__restrict__ occ,
                                                          int16_t *__restrict__ out) {
@@ -45,15 +45,20 @@ __global__ void __launch_bounds__(256) brick_aabb_kernel(const uint32_t *__restr
             c1[k] = min(b[k] * B + B, n[k]);
         }
         const int ry = c1[1] - c0[1], rows = ry * (c1[2] - c0[2]);
-        const int x0 = c0[0] + 1, w = c1[0] - c0[0];  // mask index of the first cell, width
-        const int wd = x0 >> 5, sh = x0 & 31;
-        const unsigned long long keep = (w >= 64) ? ~0ull : ((1ull << w) - 1ull);
+        const int x0 = c0[0] + 4, w = c1[0] - c0[0];  // first cell in the mask's blocks, width
+        const int nfx = cell_blocks(nx), nfy = cell_blocks(ny);
+        const int fx0 = x0 >> 2, fx1 = (x0 + w - 1) >> 2;  // blocks of 4 cells, at most 5
+        const unsigned long long keep = (1ull << w) - 1ull;
         for (int r = lane; r < rows; r += 32) {
             const int cy = c0[1] + r % ry, cz = c0[2] + r / ry;
-            const uint32_t *row = cells + ((long)(cz + 1) * (ny + 1) + (cy + 1)) * cwx;
-            unsigned long long bits = row[wd];
-            if (wd + 1 < cwx) bits |= (unsigned long long)row[wd + 1] << 32;
-            bits = (bits >> sh) & keep;
+            const int y = cy + 4, z = cz + 4;
+            const uint32_t *row =
+                cells + 2 * (((long)(z >> 2) * nfy + (y >> 2)) * nfx) + ((z >> 1) & 1);
+            unsigned long long bits = 0ull;
+            for (int fx = fx0; fx <= fx1; ++fx)
+                bits |= (unsigned long long)((row[2 * fx] >> (16 * (z & 1) + 4 * (y & 3))) & 0xfu)
+                        << (4 * (fx - fx0));
+            bits = (bits >> (x0 & 3)) & keep;
             if (bits) {
                 lo[0] = min(lo[0], c0[0] + __ffsll((long long)bits) - 1);
                 hi[0] = max(hi[0], c0[0] + 63 - __clzll((long long)bits));
@@ -214,14 +219,14 @@ int grid_for(long n, int per_block) {
 
 }  // namespace
 
-cudaError_t launch_brick_aabbs(const uint32_t *cells, int cwx, const int n[3], int B,
-                               const int nb[3], const uint8_t *occ, int16_t *out,
+cudaError_t launch_brick_aabbs(const uint32_t *cells, const int n[3], int B, const int nb[3],
+                               const uint8_t *occ, int16_t *out,
                                cudaStream_t st) {
     const long nbricks = (long)nb[0] * nb[1] * nb[2];
     const long blocks = (nbricks + 7) / 8;
     if (blocks > 0x7fffffffL) return cudaErrorInvalidValue;
-    brick_aabb_kernel<<<(unsigned)blocks, 256, 0, st>>>(cells, cwx, n[0], n[1], n[2], B, nb[0],
-                                                       nb[1], nb[2], occ, out);
+    brick_aabb_kernel<<<(unsigned)blocks, 256, 0, st>>>(cells, n[0], n[1], n[2], B, nb[0], nb[1],
+                                                       nb[2], occ, out);
     return cudaGetLastError();
 }
 

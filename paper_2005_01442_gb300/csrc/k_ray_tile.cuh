@@ -56,7 +56,6 @@ __device__ __forceinline__ void render_ray_tile(const RenderLaunch &L, int tile)
     // brick and leaves clear cells to the second phase, whose 16 lanes test 16 samples at a
     // time (testing them here, one per lane and warp step, was 1.5% slower per frame)
     const uint32_t *cells = SPLIT ? nullptr : L.cells;
-    const int cwx = L.cwx;
 
     // output pixel; in an ordered pass over pieces (L.accum) the ray continues the colour and
     // transmittance the pieces in front left there (full-image pixels, T itself), and a ray
@@ -122,8 +121,7 @@ __device__ __forceinline__ void render_ray_tile(const RenderLaunch &L, int tile)
             }
             int qs = QS_EXACT;
             if (ESL && cells && j < ray.nseg - 1) {
-                qs = quick_skip(bricks, dist, cells, cwx, gn, Pf, df, step, j, run_lin,
-                                run_empty);
+                qs = quick_skip(bricks, dist, cells, gn, Pf, df, step, j, run_lin, run_empty);
                 if (qs == QS_EMPTY_BRICK) {  // opacity zero, back to leaping
                     ++j;
                     in_run = false;
@@ -153,7 +151,7 @@ __device__ __forceinline__ void render_ray_tile(const RenderLaunch &L, int tile)
                     in_run = false;
                     continue;
                 }
-                if (cells && !cell_open(cells, cwx, gn, ip)) {  // clear cell: opacity 0
+                if (cells && !cell_open(cells, gn, ip)) {  // clear cell: opacity 0
                     ++j;
                     ++executed;
                     if (++skips == SKIP_PER_STEP) {

@@ -149,7 +149,6 @@ __global__ void __launch_bounds__(TM_THREADS, 8)
     const int gn[3] = {L.grid.n[0], L.grid.n[1], L.grid.n[2]};
     const TfView tfv = L.tf;
     const uint32_t *cells = L.cells;
-    const int cwx = L.cwx;
     const float step = L.grid.step, thr = L.grid.ert;
     const float inv_step = 1.0f / step;
 
@@ -277,7 +276,7 @@ __global__ void __launch_bounds__(TM_THREADS, 8)
                     in_run = false;
                     continue;
                 }
-                if (cells && !cell_open(cells, cwx, gn, ip)) {
+                if (cells && !cell_open(cells, gn, ip)) {
                     ++j;
                     ++executed;
                     continue;

@@ -32,7 +32,7 @@ struct Occ {
     uint8_t *dev = nullptr;   // occupancy bytes
     uint8_t *dist = nullptr;  // 8 forward-box distance fields (0 = occupied)
     int *scratch = nullptr;   // summed-volume table used while building dist
-    uint32_t *cells = nullptr;  // cell transparency mask (cellmask_words words)
+    uint32_t *cells = nullptr;  // cell transparency mask (cellmask_bytes)
     long n = 0;
     unsigned brick_version = 0, tf_version = 0;
     int16_t *aabb = nullptr;    // tight visible box per brick (6 int16), built on first use
@@ -45,7 +45,6 @@ struct Volume {
     int pnx = 0, pny = 0, pnz = 0;
     void *dpad = nullptr;          // compact padded copy (brick tables)
     float4 *drep = nullptr;        // x-replicated float4 copy (rendering)
-    uint8_t *mask_scratch = nullptr;  // cell-mask build scratch (cellmask_scratch_bytes)
     float *dpadf = nullptr;           // float32 copy of dpad (TMA-staged render), on first use
     struct alignas(64) { unsigned char b[128]; } tmap;  // tensor map of dpadf
     Bricks bricks[2];               // B = 8, B = 16
@@ -169,7 +168,6 @@ void free_volume(Volume &v) {
     cudaFree(v.dpad);
     cudaFree(v.dpadf);
     cudaFree(v.drep);
-    cudaFree(v.mask_scratch);
     for (auto &b : v.bricks) {
         cudaFree(b.mn);
         cudaFree(b.mx);
@@ -375,8 +373,7 @@ vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStre
         CK(cudaMalloc(&o.dev, (size_t)b.count()), "cudaMalloc(occupancy)");
         CK(cudaMalloc(&o.dist, 8 * (size_t)b.count()), "cudaMalloc(occupancy)");
         CK(cudaMalloc(&o.scratch, box_dist_scratch_bytes(b.nb)), "cudaMalloc(occupancy)");
-        CK(cudaMalloc(&o.cells, sizeof(uint32_t) * (size_t)cellmask_words(v.n)),
-           "cudaMalloc(cell mask)");
+        CK(cudaMalloc(&o.cells, cellmask_bytes(v.n)), "cudaMalloc(cell mask)");
         o.n = b.count();
         o.brick_version = o.tf_version = 0;
     }
@@ -384,10 +381,7 @@ vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStre
         CK(launch_occupancy(b.mn, b.mx, v.dtype, b.count(), t.prefix, t.lo, t.du, o.dev, st),
            "occupancy launch");
         CK(launch_box_dist(o.dev, b.nb, o.scratch, o.dist, st), "distance launch");
-        if (!v.mask_scratch)
-            CK(cudaMalloc(&v.mask_scratch, cellmask_scratch_bytes(view_of(v))),
-               "cudaMalloc(cell mask scratch)");
-        CK(launch_cellmask(view_of(v), t.zrun, t.lo, t.du, v.mask_scratch, o.cells, st),
+        CK(launch_cellmask(view_of(v), B, b.nb, o.dev, t.zrun, t.lo, t.du, o.cells, st),
            "cell mask launch");
         o.brick_version = b.version;
         o.tf_version = t.version;
@@ -412,7 +406,7 @@ vrc_status ensure_aabb(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStr
         o.aabb_brick_version = o.aabb_tf_version = 0;
     }
     if (o.aabb_brick_version != o.brick_version || o.aabb_tf_version != o.tf_version) {
-        CK(launch_brick_aabbs(cells, (v.n[0] + 1 + 31) / 32, v.n, B, b.nb, occ, o.aabb, st),
+        CK(launch_brick_aabbs(cells, v.n, B, b.nb, occ, o.aabb, st),
            "box launch");
         o.aabb_brick_version = o.brick_version;
         o.aabb_tf_version = o.tf_version;
@@ -604,7 +598,6 @@ vrc_status prepare_render(vrc_ctx *ctx, int vol_id, int tf_id, const vrc_camera 
         Bricks &b = v->bricks[slot_of(p->brick)];
         L.dist = dist;
         L.cells = cells;
-        L.cwx = (v->n[0] + 1 + 31) / 32;
         L.bricks.B = b.B;
         L.bricks.shift = b.B == 16 ? 4 : 3;
         L.bricks.margin = leap_margin(v->n);
@@ -998,17 +991,23 @@ vrc_status vrc_cellmask_get(vrc_ctx *ctx, int vol_id, int tf_id, int B, uint32_t
     Tf *t = get_tf(ctx, tf_id);
     if (!t) return fail(ctx, VRC_ERR_ARG, "unknown transfer function id %d", tf_id);
     if (B != 8 && B != 16) return fail(ctx, VRC_ERR_ARG, "brick must be 8 or 16");
-    if (nwords != cellmask_words(v->n))
-        return fail(ctx, VRC_ERR_ARG, "nwords must be %ld", cellmask_words(v->n));
+    if (nwords != cellmask_row_words(v->n))
+        return fail(ctx, VRC_ERR_ARG, "nwords must be %ld", cellmask_row_words(v->n));
     DeviceGuard g(ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const uint8_t *occ = nullptr;
     const uint32_t *cells = nullptr;
     vrc_status s = ensure_occ(ctx, *v, tf_id, *t, B, st, &occ, nullptr, &cells);
     if (s != VRC_OK) return s;
-    CK(cudaMemcpyAsync(words_host, cells, sizeof(uint32_t) * (size_t)nwords,
-                       cudaMemcpyDeviceToHost, st), "cell mask copy");
-    CK(cudaStreamSynchronize(st), "cell mask copy sync");
+    uint32_t *rows = nullptr;
+    cudaError_t e = cudaMalloc(&rows, sizeof(uint32_t) * (size_t)nwords);
+    if (e == cudaSuccess) e = launch_cellmask_rows(cells, v->n, rows, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(words_host, rows, sizeof(uint32_t) * (size_t)nwords,
+                            cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFree(rows);
+    CK(e, "cell mask copy");
     return VRC_OK;
 }
 
@@ -1363,15 +1362,12 @@ extern "C" vrc_status vrc_render_noalloc(vrc_ctx *ctx, int vol_id, int tf_id,
         CK(launch_occupancy(b->mn, b->mx, v->dtype, b->count(), t->prefix, t->lo, t->du, occ, st),
            "occupancy launch");
         CK(launch_box_dist(occ, b->nb, svt, dist, st), "distance launch");
-        // the cell mask too when it and its build scratch fit behind the tables (it only
-        // saves work)
-        const size_t mask_off = cells_off + align256(sizeof(uint32_t) * (size_t)cellmask_words(v->n));
-        if (mask_off + cellmask_scratch_bytes(view_of(*v)) <= (size_t)VRC_NOALLOC_SCRATCH_BYTES) {
+        // the cell mask too when it fits behind the tables (it only saves work)
+        if (cells_off + cellmask_bytes(v->n) <= (size_t)VRC_NOALLOC_SCRATCH_BYTES) {
             uint32_t *cells = (uint32_t *)(scratch + cells_off);
-            CK(launch_cellmask(view_of(*v), t->zrun, t->lo, t->du, scratch + mask_off, cells, st),
+            CK(launch_cellmask(view_of(*v), B, b->nb, occ, t->zrun, t->lo, t->du, cells, st),
                "cell mask launch");
             L.cells = cells;
-            L.cwx = (v->n[0] + 1 + 31) / 32;
         }
         L.dist = dist;
         L.bricks.B = b->B;

@@ -410,7 +410,6 @@ struct RenderLaunch {
     int *err;                      // device error word
     RaySplit split;                // used by the split render only
     const uint32_t *cells;         // NULL, or the cell transparency mask (with dist)
-    int cwx;                       // mask words per row of cells along x
     int mode;                      // interpolation / classification variant (MODE_*)
     Phong phong;                   // MODE_CUBIC_PHONG only
     const float4 *preint;          // MODE_PREINT only: the table for slabs of length step
@@ -446,12 +445,22 @@ inline int ckpt_segments(const int n[3], float step, int seg) {
     return (int)__builtin_ceil(samples / (double)seg);
 }
 
+// Cell transparency mask: cells c = -1 .. n-1 per axis in blocks of 4^3, cell c in block
+// (c + 4) >> 2 (blocks do not straddle bricks; block 0 holds the cells -1), block
+// (bz * cell_blocks(ny) + by) * cell_blocks(nx) + bx, two 32-bit words per block (c_z & 2 picks
+// the word), bit 16 (c_z & 1) + 4 (c_y & 3) + (c_x & 3). A ray's next samples mostly fall into
+// the word it read last, and 32 bytes hold a run of 4 blocks. A tile is 2^3 blocks: cell c in
+// tile (c + 8) >> 3.
+VRC_HD int cell_blocks(int n) { return ((n + 3) >> 2) + 1; }
+VRC_HD int cell_tiles(int n) { return ((n + 7) >> 3) + 1; }
+
 // Bit of the cell holding sample base ip (ip in [-1, n-1]); 0: the sample's opacity is zero.
-__device__ __forceinline__ bool cell_open(const uint32_t *__restrict__ cells, int cwx,
-                                          const int n[3], const int ip[3]) {
-    const int cx = ip[0] + 1, cy = ip[1] + 1, cz = ip[2] + 1;
-    const uint32_t w = __ldg(cells + ((long)cz * (n[1] + 1) + cy) * cwx + (cx >> 5));
-    return (w >> (cx & 31)) & 1u;
+__device__ __forceinline__ bool cell_open(const uint32_t *__restrict__ cells, const int n[3],
+                                          const int ip[3]) {
+    const int cx = ip[0] + 4, cy = ip[1] + 4, cz = ip[2] + 4;
+    const int blk = ((cz >> 2) * cell_blocks(n[1]) + (cy >> 2)) * cell_blocks(n[0]) + (cx >> 2);
+    const uint32_t w = __ldg(cells + 2 * blk + ((cz >> 1) & 1));
+    return (w >> (((cz & 1) << 4) | ((cy & 3) << 2) | (cx & 3))) & 1u;
 }
 
 // Quick skip test of sample j < nseg - 1 from its float position (the leap path's, within a
@@ -462,9 +471,9 @@ __device__ __forceinline__ bool cell_open(const uint32_t *__restrict__ cells, in
 // Without a cell mask (cells == NULL) only the brick is tested.
 enum { QS_EXACT = 0, QS_EMPTY_BRICK = 1, QS_CLEAR_CELL = 2, QS_OPEN = 3 };
 __device__ __forceinline__ int quick_skip(const BrickView &bv, const uint8_t *__restrict__ dist,
-                                          const uint32_t *__restrict__ cells, int cwx,
-                                          const int n[3], const float Pf[3], const float df[3],
-                                          float step, int j, int &cache_lin, int &cache_empty) {
+                                          const uint32_t *__restrict__ cells, const int n[3],
+                                          const float Pf[3], const float df[3], float step,
+                                          int j, int &cache_lin, int &cache_empty) {
     const float m = ((float)j + 0.5f) * step;
     int c[3];
     bool near = false;
@@ -485,7 +494,7 @@ __device__ __forceinline__ int quick_skip(const BrickView &bv, const uint8_t *__
     }
     if (cache_empty) return QS_EMPTY_BRICK;
     if (!cells) return QS_OPEN;
-    return cell_open(cells, cwx, n, c) ? QS_OPEN : QS_CLEAR_CELL;
+    return cell_open(cells, n, c) ? QS_OPEN : QS_CLEAR_CELL;
 }
 
 // Launchers (return cudaSuccess or the launch error).
@@ -497,14 +506,17 @@ cudaError_t launch_brick_minmax(const VolView &v, int B, void *mn, void *mx, cud
 cudaError_t launch_occupancy(const void *mn, const void *mx, int dtype, long nbricks,
                              const int *prefix_dev, float lo, float du, uint8_t *occ,
                              cudaStream_t st);
-// Cell transparency mask of a padded volume for a transfer function, given the run id of
-// each zero-opacity table entry (1, 2, ... per maximal run of zero entries; 0 for entries of
-// non-zero opacity): cellmask_words(n) words.
-// `scratch` holds cellmask_scratch_bytes(v) bytes (16-byte aligned) for the build.
-long cellmask_words(const int n[3]);
-size_t cellmask_scratch_bytes(const VolView &v);
-cudaError_t launch_cellmask(const VolView &v, const uint8_t *zrun_dev, float lo, float du,
-                            uint8_t *scratch, uint32_t *cells, cudaStream_t st);
+// Cell transparency mask of a padded volume for a transfer function (layout: cell_open), given
+// its occupancy with bricks of size B and the run id of each zero-opacity table entry (1, 2,
+// ... per maximal run of zero entries; 0 for entries of non-zero opacity).
+size_t cellmask_bytes(const int n[3]);
+cudaError_t launch_cellmask(const VolView &v, int B, const int nb[3], const uint8_t *occ,
+                            const uint8_t *zrun_dev, float lo, float du, uint32_t *cells,
+                            cudaStream_t st);
+// The mask as rows of 32-cell words along x, the layout vrc_cellmask_get returns.
+long cellmask_row_words(const int n[3]);
+cudaError_t launch_cellmask_rows(const uint32_t *cells, const int n[3], uint32_t *out,
+                                 cudaStream_t st);
 size_t box_dist_scratch_bytes(const int nb[3]);
 // dist: 8 x nbricks bytes (one forward-box distance field per direction octant)
 cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], int *scratch, uint8_t *dist,
@@ -519,8 +531,8 @@ struct CompositeArgs {
     int rect[MAX_PIECES][4];
 };
 // out: 6 int16 per brick (tight visible box, half-open cell coordinates, zeros when empty)
-cudaError_t launch_brick_aabbs(const uint32_t *cells, int cwx, const int n[3], int B,
-                               const int nb[3], const uint8_t *occ, int16_t *out,
+cudaError_t launch_brick_aabbs(const uint32_t *cells, const int n[3], int B, const int nb[3],
+                               const uint8_t *occ, int16_t *out,
                                cudaStream_t st);
 cudaError_t launch_piece_mask(const uint8_t *occ, const int nb[3], const int blo[3],
                               const int bhi[3], uint8_t *out, cudaStream_t st);
