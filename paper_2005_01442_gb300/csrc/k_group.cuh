@@ -3,7 +3,7 @@
 //
 // The ray is walked in blocks of G consecutive sample indices, lane q of the group taking
 // sample G k + q. Every lane places its sample exactly from the double-float ray record,
-// resamples the uniform cubic B-spline from the x-replicated float4 volume, classifies it
+// resamples the uniform cubic B-spline from the render layout (ReplView), classifies it
 // through the transfer function and corrects its opacity to the segment length (paper, Sec.
 // "Methodology": cubic interpolation, post-classification). The block is composited front to
 // back by a group-wide inclusive scan of the "over" operator

@@ -4,7 +4,7 @@
 // cubic interpolation with post-classification is preferred).
 //
 // Per sample: exact placement from the double-float ray record, the 64-tap uniform cubic
-// B-spline read as 16 aligned float4 rows of the x-replicated volume through L1,
+// B-spline read from the render layout (ReplView) through L1,
 // post-classification through the 256-entry table, opacity corrected to the segment length,
 // front-to-back compositing, early ray termination. With a brick table the ray leaps over
 // boxes of empty bricks ahead of it (Sec. "Analysis", Pros (b): auxiliary structures to skip

@@ -3,7 +3,7 @@
 // A CTA renders an 8 x 8 pixel tile, one ray per thread (paper, Sec. "Methodology": one ray
 // per pixel, fixed step, cubic interpolation, post-classification, front-to-back
 // accumulation). Neighbouring rays read largely the same voxels, so instead of every thread
-// gathering its 64 taps through L1 from the x-replicated float4 layout (16 bytes per voxel,
+// gathering its 64 taps through L1 from the render layout (ReplView, 16 bytes per voxel,
 // mostly L2 misses once rays are long), the CTA copies the part of the volume its rays will
 // sample next into shared memory once and all threads resample from there:
 //
@@ -22,7 +22,7 @@
 //      skipped, and the exact test decides the same way).
 //
 // Windows whose box does not fit (a tile that covers many voxels: small images, close-up
-// perspective) are resampled through L1 from the x-replicated layout instead; both paths
+// perspective) are resampled through L1 from the render layout instead; both paths
 // compute the same sums in the same order, so the image equals the per-ray kernel's bit for
 // bit. The staged box lies inside the padded volume (taps reach -2 .. n+1) except past its
 // far faces, where the copy fills zeros that no tap reads.

@@ -44,7 +44,7 @@ struct Volume {
     int n[3] = {0, 0, 0};
     int pnx = 0, pny = 0, pnz = 0;
     void *dpad = nullptr;          // compact padded copy (brick tables)
-    float4 *drep = nullptr;        // x-replicated float4 copy (rendering)
+    void *drep = nullptr;          // render layout (ReplView)
     float *dpadf = nullptr;           // float32 copy of dpad (TMA-staged render), on first use
     struct alignas(64) { unsigned char b[128]; } tmap;  // tensor map of dpadf
     Bricks bricks[2];               // B = 8, B = 16
@@ -557,10 +557,7 @@ vrc_status prepare_render(vrc_ctx *ctx, int vol_id, int tf_id, const vrc_camera 
     vrc_status s = build_camera(ctx, cam, L.cam);
     if (s != VRC_OK) return s;
     L.vol = view_of(*v);
-    L.rep.base = v->drep;
-    L.rep.rnx = v->n[0] + 1;
-    L.rep.rny = v->n[1] + 4;
-    L.rep.rnz = v->n[2] + 4;
+    L.rep = rep_view(v->drep, v->dtype, v->n);
     L.tf = tf_view(*t);
     L.phong.eps = 0.01f * (t->hi - t->lo);
     for (int k = 0; k < 3; ++k) L.grid.n[k] = v->n[k];
@@ -786,10 +783,8 @@ vrc_status vrc_volume_upload(vrc_ctx *ctx, const void *data, int on_device, vrc_
         if (e == cudaSuccess) e = cudaMemcpyAsync(staging, data, raw, cudaMemcpyHostToDevice, st);
         src = staging;
     }
-    const size_t rep = (size_t)(nx + 1) * (ny + 4) * (nz + 4) * sizeof(float4);
-    if (e == cudaSuccess) e = cudaMalloc(&v.drep, rep);
-    if (e == cudaSuccess) e = launch_pad_volume(src, dtype, v.n, v.dpad, v.pnx, v.pny, v.pnz, st);
-    if (e == cudaSuccess) e = launch_replicate_x4(src, dtype, v.n, v.drep, st);
+    if (e == cudaSuccess) e = cudaMalloc(&v.drep, rep_bytes(dtype, v.n));
+    if (e == cudaSuccess) e = launch_volume_layouts(src, dtype, v.n, v.dpad, v.pnx, v.drep, st);
     if (staging) {
         cudaError_t e2 = cudaStreamSynchronize(st);
         if (e == cudaSuccess) e = e2;
@@ -823,8 +818,8 @@ vrc_status vrc_volume_update(vrc_ctx *ctx, int vol_id, const void *data, int on_
         if (e == cudaSuccess) e = cudaMemcpyAsync(staging, data, raw, cudaMemcpyHostToDevice, st);
         src = staging;
     }
-    if (e == cudaSuccess) e = launch_pad_volume(src, v->dtype, v->n, v->dpad, v->pnx, v->pny, v->pnz, st);
-    if (e == cudaSuccess) e = launch_replicate_x4(src, v->dtype, v->n, v->drep, st);
+    if (e == cudaSuccess)
+        e = launch_volume_layouts(src, v->dtype, v->n, v->dpad, v->pnx, v->drep, st);
     if (e == cudaSuccess && v->dpadf) e = launch_padded_to_float(view_of(*v), v->dpadf, st);
     if (staging) {
         cudaError_t e2 = cudaStreamSynchronize(st);

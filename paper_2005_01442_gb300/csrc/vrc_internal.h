@@ -28,11 +28,28 @@ struct VolView {
     int pnx, pny, pnz;
 };
 
-// The render layout of a resident volume (float4 entries replicated along x, see
-// replicate_x4_kernel): rnx = nx + 1, rny = ny + 4, rnz = nz + 4.
+// The render layout of a resident volume: 16-byte entries, each voxel in several of them, so
+// that a sample reads its 64 taps with few aligned 16-byte loads. Indices are clamped to the
+// volume (clamp-to-edge) when the layout is written.
+//
+// float32: entry (x', y', z') holds the voxels x'-2 .. x'+1 of row (y'-2, z'-2); x' in [0, nx],
+//   y' in [0, ny+3], z' in [0, nz+3]. A sample at base i reads entries (i0+1, i1+1+b, i2+1+c),
+//   16 loads.
+// 16-bit: entry (x', y', z') holds the 2^3 voxels from (x'-2, y'-2, z'-2): four words, one per
+//   (x, y) with x fastest, low half the lower z, each voxel plus `bias` as an unsigned 16-bit
+//   value; x' in [0, nx+2] and so on. Along x the entries of even x' come first, then those of
+//   odd x' (`half` of each per row), since a sample reads entries of one parity: (i0+1 + {0, 2},
+//   i1+1 + {0, 2}, i2+1 + {0, 2}), 8 loads, pairs of them adjacent.
+//   Half the loads and bytes of the same volume as float4 rows: a dense 1024^2 frame of a 512^2
+//   x 400 CT was bound by the L1 data path (93% of its peak, 934 M wavefronts) and takes 2.79 ms
+//   (706 M) instead of 3.15; unpacking costs 96 instructions a sample, of which packed float32
+//   arithmetic saves 40 again. Float32 volumes keep the rows of 4: packing them by z would save
+//   the 40 but no load.
 struct ReplView {
-    const float4 *base;
-    int rnx, rny, rnz;
+    const void *base;
+    int rnx, rny;   // entries per row, rows per slice
+    int half;       // 16-bit: entries of each parity per row; 0: float32
+    float magic;    // 16-bit: 2^23 + bias
 };
 
 // Brick table of size B (min/max arrays of the voxel dtype, ceil(n/B) per axis).
@@ -117,20 +134,144 @@ __device__ __forceinline__ int leap_float(const BrickView &bv, const uint8_t *__
     return max(jn, j + 1);
 }
 
-// Cubic B-spline sample at integer base ip (taps ip-1 .. ip+2) with fractions f, from the
-// x-replicated float4 volume: entry (ip0 + 1, ip1 + 1 + b, ip2 + 1 + c) holds tap row (b, c).
+// Two float32 in one 64-bit register pair, with the packed arithmetic of sm_100 (each half
+// rounded on its own, as the scalar operations).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// The two 16-bit values of a word as float32, exactly: 2^23 + u by byte insertion, minus 2^23 +
+// bias (sub = the pair of -(2^23 + bias)).
+__device__ __forceinline__ f32x2 voxels2(uint32_t w, f32x2 sub) {
+    return add2(pack2(__uint_as_float(__byte_perm(w, 0x4b00u, 0x5410)),
+                      __uint_as_float(__byte_perm(w, 0x4b00u, 0x5432))),
+                sub);
+}
+
+// 16-bit layout: entry of voxels (x, y, z) .. + 1, x >= -2 and so on.
+__device__ __forceinline__ const uint4 *entry16(const ReplView &rp, int x, int y, int z) {
+    x += 2;
+    const unsigned i = ((unsigned)(z + 2) * rp.rny + (unsigned)(y + 2)) * rp.rnx +
+                       ((x & 1) ? rp.half : 0) + (x >> 1);
+    return (const uint4 *)rp.base + i;
+}
+
+__device__ __forceinline__ const float4 *entry32(const ReplView &rp, int x, int y, int z) {
+    const unsigned i = ((unsigned)(z + 2) * rp.rny + (unsigned)(y + 2)) * rp.rnx +
+                       (unsigned)(x + 2);
+    return (const float4 *)rp.base + i;
+}
+
+// Calls fn(c, b, v) for the 16 tap rows (y ip1-1+b, z ip2-1+c) of base ip, c outermost; v holds
+// the voxels ip0-1 .. ip0+2 of the row.
+template <class Fn>
+__device__ __forceinline__ void for_rows(const ReplView &rp, const int ip[3], Fn fn) {
+    if (rp.half) {
+        const f32x2 sub = pack2(-rp.magic, -rp.magic);
+        const uint4 *p = entry16(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+        const unsigned row2 = 2u * rp.rnx, slice2 = row2 * rp.rny;
+#pragma unroll
+        for (int zh = 0; zh < 2; ++zh) {
+            float4 v[2][4];  // rows of the lower and the upper z
+#pragma unroll
+            for (int yh = 0; yh < 2; ++yh) {
+                const uint4 *e = p + (zh ? slice2 : 0u) + (yh ? row2 : 0u);
+                const uint4 a = __ldg(e), b = __ldg(e + 1);
+                const float2 a0 = unpack2(voxels2(a.x, sub)), a1 = unpack2(voxels2(a.y, sub));
+                const float2 a2 = unpack2(voxels2(a.z, sub)), a3 = unpack2(voxels2(a.w, sub));
+                const float2 b0 = unpack2(voxels2(b.x, sub)), b1 = unpack2(voxels2(b.y, sub));
+                const float2 b2 = unpack2(voxels2(b.z, sub)), b3 = unpack2(voxels2(b.w, sub));
+                v[0][2 * yh] = make_float4(a0.x, a1.x, b0.x, b1.x);
+                v[1][2 * yh] = make_float4(a0.y, a1.y, b0.y, b1.y);
+                v[0][2 * yh + 1] = make_float4(a2.x, a3.x, b2.x, b3.x);
+                v[1][2 * yh + 1] = make_float4(a2.y, a3.y, b2.y, b3.y);
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) fn(2 * zh + h, b, v[h][b]);
+        }
+    } else {
+        const float4 *p = entry32(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+        const unsigned slice = (unsigned)rp.rnx * rp.rny;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) fn(c, b, __ldg(p + c * slice + b * rp.rnx));
+    }
+}
+
+// Cubic B-spline sample at integer base ip (taps ip-1 .. ip+2) with fractions f. Both layouts
+// sum the same products in the same order: along x, then y, then z.
 __device__ __forceinline__ float tricubic_rep(const ReplView &rp, const int ip[3],
                                               const float f[3]) {
     float wx[4], wy[4], wz[4];
     bspline_w(f[0], wx);
     bspline_w(f[1], wy);
     bspline_w(f[2], wz);
-    const long rslice = (long)rp.rnx * rp.rny;
-    const float4 *p0 = rp.base + ((long)(ip[2] + 1) * rp.rny + (ip[1] + 1)) * rp.rnx + (ip[0] + 1);
     float s = 0.0f;
+    if (rp.half) {
+        // two z at a time
+        const f32x2 sub = pack2(-rp.magic, -rp.magic);
+        f32x2 wx2[4], wy2[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            wx2[k] = pack2(wx[k], wx[k]);
+            wy2[k] = pack2(wy[k], wy[k]);
+        }
+        const uint4 *p = entry16(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+        const unsigned row2 = 2u * rp.rnx, slice2 = row2 * rp.rny;
+        uint4 e[2][2][2];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            e[k >> 2][(k >> 1) & 1][k & 1] =
+                __ldg(p + ((k & 4) ? slice2 : 0u) + ((k & 2) ? row2 : 0u) + (k & 1));
+#pragma unroll
+        for (int zh = 0; zh < 2; ++zh) {
+            f32x2 plane = 0ull;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const uint4 l = e[zh][b >> 1][0], u = e[zh][b >> 1][1];
+                f32x2 r = mul2(wx2[0], voxels2((b & 1) ? l.z : l.x, sub));
+                r = fma2(wx2[1], voxels2((b & 1) ? l.w : l.y, sub), r);
+                r = fma2(wx2[2], voxels2((b & 1) ? u.z : u.x, sub), r);
+                r = fma2(wx2[3], voxels2((b & 1) ? u.w : u.y, sub), r);
+                plane = fma2(wy2[b], r, plane);
+            }
+            const float2 pl = unpack2(plane);
+            s = fmaf(wz[2 * zh], pl.x, s);
+            s = fmaf(wz[2 * zh + 1], pl.y, s);
+        }
+        return s;
+    }
+    const float4 *p0 = entry32(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+    const unsigned slice = (unsigned)rp.rnx * rp.rny;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float4 *pc = p0 + c * rslice;
+        const float4 *pc = p0 + c * slice;
         float plane = 0.0f;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
@@ -171,18 +312,37 @@ __device__ __forceinline__ float4 preint_lookup(const float4 *__restrict__ tab, 
     return o;
 }
 
-// Trilinear sample at integer base ip (taps ip .. ip+1, clamped) with fractions f, from the
-// x-replicated float4 volume: entry (ip0 + 1, ip1 + 1 + b, ip2 + 1 + c) for b, c in {1, 2},
-// components y and z (voxels ip0 and ip0 + 1).
+// The 8 voxels ip .. ip+1 (clamped), x fastest, then y, then z.
+__device__ __forceinline__ void taps8(const ReplView &rp, const int ip[3], float v[8]) {
+    if (rp.half) {
+        const f32x2 sub = pack2(-rp.magic, -rp.magic);
+        const uint4 e = __ldg(entry16(rp, ip[0], ip[1], ip[2]));
+        const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 z = unpack2(voxels2(w[k], sub));
+            v[k] = z.x;
+            v[k + 4] = z.y;
+        }
+        return;
+    }
+    const float4 *p = entry32(rp, ip[0] - 1, ip[1], ip[2]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // components y and z: voxels ip0 and ip0 + 1
+        const float4 r = __ldg(p + (k >> 1) * ((unsigned)rp.rnx * rp.rny) + (k & 1) * rp.rnx);
+        v[2 * k] = r.y;
+        v[2 * k + 1] = r.z;
+    }
+}
+
+// Trilinear sample at integer base ip with fractions f.
 __device__ __forceinline__ float trilinear_rep(const ReplView &rp, const int ip[3],
                                                const float f[3]) {
-    const long rslice = (long)rp.rnx * rp.rny;
-    const float4 *p0 = rp.base + ((long)(ip[2] + 2) * rp.rny + (ip[1] + 2)) * rp.rnx + (ip[0] + 1);
-    const float4 a = __ldg(p0), b = __ldg(p0 + rp.rnx);
-    const float4 c = __ldg(p0 + rslice), d = __ldg(p0 + rslice + rp.rnx);
+    float v[8];
+    taps8(rp, ip, v);
     const float gx = 1.0f - f[0], gy = 1.0f - f[1], gz = 1.0f - f[2];
-    const float r0 = fmaf(f[0], a.z, gx * a.y), r1 = fmaf(f[0], b.z, gx * b.y);
-    const float r2 = fmaf(f[0], c.z, gx * c.y), r3 = fmaf(f[0], d.z, gx * d.y);
+    const float r0 = fmaf(f[0], v[1], gx * v[0]), r1 = fmaf(f[0], v[3], gx * v[2]);
+    const float r2 = fmaf(f[0], v[5], gx * v[4]), r3 = fmaf(f[0], v[7], gx * v[6]);
     const float q0 = fmaf(f[1], r1, gy * r0), q1 = fmaf(f[1], r3, gy * r2);
     return fmaf(f[2], q1, gz * q0);
 }
@@ -206,7 +366,7 @@ struct Phong {
 };
 
 // Value and gradient of the cubic B-spline at integer base ip with fractions f (derivative
-// weights d/df of the weights, the same 16 float4 rows).
+// weights d/df of the weights, the same taps).
 __device__ __forceinline__ float tricubic_grad_rep(const ReplView &rp, const int ip[3],
                                                    const float f[3], float g[3]) {
     float wx[4], wy[4], wz[4], dx[4], dy[4], dz[4];
@@ -216,34 +376,72 @@ __device__ __forceinline__ float tricubic_grad_rep(const ReplView &rp, const int
     bspline_dw(f[0], dx);
     bspline_dw(f[1], dy);
     bspline_dw(f[2], dz);
-    const long rslice = (long)rp.rnx * rp.rny;
-    const float4 *p0 = rp.base + ((long)(ip[2] + 1) * rp.rny + (ip[1] + 1)) * rp.rnx + (ip[0] + 1);
     float s = 0.0f;
     g[0] = g[1] = g[2] = 0.0f;
+    if (rp.half) {  // two z at a time, as in tricubic_rep
+        const f32x2 sub = pack2(-rp.magic, -rp.magic);
+        f32x2 wx2[4], dx2[4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float4 *pc = p0 + c * rslice;
-        float ps = 0.0f, pdx = 0.0f, pdy = 0.0f;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const float4 v = __ldg(pc + b * rp.rnx);
-            float r = wx[0] * v.x;
-            r = fmaf(wx[1], v.y, r);
-            r = fmaf(wx[2], v.z, r);
-            r = fmaf(wx[3], v.w, r);
-            float rd = dx[0] * v.x;
-            rd = fmaf(dx[1], v.y, rd);
-            rd = fmaf(dx[2], v.z, rd);
-            rd = fmaf(dx[3], v.w, rd);
-            ps = fmaf(wy[b], r, ps);
-            pdx = fmaf(wy[b], rd, pdx);
-            pdy = fmaf(dy[b], r, pdy);
+        for (int k = 0; k < 4; ++k) {
+            wx2[k] = pack2(wx[k], wx[k]);
+            dx2[k] = pack2(dx[k], dx[k]);
         }
+        const uint4 *p = entry16(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+        const unsigned row2 = 2u * rp.rnx, slice2 = row2 * rp.rny;
+#pragma unroll
+        for (int zh = 0; zh < 2; ++zh) {
+            f32x2 ps = 0ull, pdx = 0ull, pdy = 0ull;
+#pragma unroll
+            for (int yh = 0; yh < 2; ++yh) {
+                const uint4 *e = p + (zh ? slice2 : 0u) + (yh ? row2 : 0u);
+                const uint4 l = __ldg(e), u = __ldg(e + 1);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int b = 2 * yh + k;
+                    const f32x2 v0 = voxels2(k ? l.z : l.x, sub), v1 = voxels2(k ? l.w : l.y, sub);
+                    const f32x2 v2 = voxels2(k ? u.z : u.x, sub), v3 = voxels2(k ? u.w : u.y, sub);
+                    const f32x2 r =
+                        fma2(wx2[3], v3, fma2(wx2[2], v2, fma2(wx2[1], v1, mul2(wx2[0], v0))));
+                    const f32x2 rd =
+                        fma2(dx2[3], v3, fma2(dx2[2], v2, fma2(dx2[1], v1, mul2(dx2[0], v0))));
+                    const f32x2 wyb = pack2(wy[b], wy[b]);
+                    ps = fma2(wyb, r, ps);
+                    pdx = fma2(wyb, rd, pdx);
+                    pdy = fma2(pack2(dy[b], dy[b]), r, pdy);
+                }
+            }
+            const float2 p0 = unpack2(ps), p1 = unpack2(pdx), p2 = unpack2(pdy);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = 2 * zh + h;
+                s = fmaf(wz[c], h ? p0.y : p0.x, s);
+                g[0] = fmaf(wz[c], h ? p1.y : p1.x, g[0]);
+                g[1] = fmaf(wz[c], h ? p2.y : p2.x, g[1]);
+                g[2] = fmaf(dz[c], h ? p0.y : p0.x, g[2]);
+            }
+        }
+        return s;
+    }
+    float ps = 0.0f, pdx = 0.0f, pdy = 0.0f;
+    for_rows(rp, ip, [&](int c, int b, const float4 &v) {
+        float r = wx[0] * v.x;
+        r = fmaf(wx[1], v.y, r);
+        r = fmaf(wx[2], v.z, r);
+        r = fmaf(wx[3], v.w, r);
+        float rd = dx[0] * v.x;
+        rd = fmaf(dx[1], v.y, rd);
+        rd = fmaf(dx[2], v.z, rd);
+        rd = fmaf(dx[3], v.w, rd);
+        ps = fmaf(wy[b], r, ps);
+        pdx = fmaf(wy[b], rd, pdx);
+        pdy = fmaf(dy[b], r, pdy);
+        if (b < 3) return;
         s = fmaf(wz[c], ps, s);
         g[0] = fmaf(wz[c], pdx, g[0]);
         g[1] = fmaf(wz[c], pdy, g[1]);
         g[2] = fmaf(dz[c], ps, g[2]);
-    }
+        ps = pdx = pdy = 0.0f;
+    });
     return s;
 }
 
@@ -287,47 +485,34 @@ __device__ __forceinline__ float4 sample_rgba(const ReplView &rp, const TfView &
         bspline_w(f[0], wx);
         bspline_w(f[1], wy);
         bspline_w(f[2], wz);
-        const long rslice = (long)rp.rnx * rp.rny;
-        const float4 *p0 =
-            rp.base + ((long)(ip[2] + 1) * rp.rny + (ip[1] + 1)) * rp.rnx + (ip[0] + 1);
         float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        for (int c = 0; c < 4; ++c) {
+        for_rows(rp, ip, [&](int c, int b, const float4 &v) {
+            const float vals[4] = {v.x, v.y, v.z, v.w};
+            const float wyz = wy[b] * wz[c];
 #pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const float4 v = __ldg(p0 + c * rslice + b * rp.rnx);
-                const float vals[4] = {v.x, v.y, v.z, v.w};
-                const float wyz = wy[b] * wz[c];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const float4 t = tf_classify(tf, vals[a]);
-                    const float w = wx[a] * wyz;
-                    acc.x = fmaf(w, t.x, acc.x);
-                    acc.y = fmaf(w, t.y, acc.y);
-                    acc.z = fmaf(w, t.z, acc.z);
-                    acc.w = fmaf(w, t.w, acc.w);
-                }
+            for (int a = 0; a < 4; ++a) {
+                const float4 t = tf_classify(tf, vals[a]);
+                const float w = wx[a] * wyz;
+                acc.x = fmaf(w, t.x, acc.x);
+                acc.y = fmaf(w, t.y, acc.y);
+                acc.z = fmaf(w, t.z, acc.z);
+                acc.w = fmaf(w, t.w, acc.w);
             }
-        }
+        });
         return acc;
     } else {
-        const long rslice = (long)rp.rnx * rp.rny;
-        const float4 *p0 =
-            rp.base + ((long)(ip[2] + 2) * rp.rny + (ip[1] + 2)) * rp.rnx + (ip[0] + 1);
-        const float w1[3] = {f[0], f[1], f[2]};
+        float v[8];
+        taps8(rp, ip, v);
         float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                const float4 v = __ldg(p0 + c * rslice + b * rp.rnx);
-                const float wyz = (b ? w1[1] : 1.0f - w1[1]) * (c ? w1[2] : 1.0f - w1[2]);
-                const float4 t0 = tf_classify(tf, v.y), t1 = tf_classify(tf, v.z);
-                const float wa = (1.0f - w1[0]) * wyz, wb = w1[0] * wyz;
-                acc.x = fmaf(wb, t1.x, fmaf(wa, t0.x, acc.x));
-                acc.y = fmaf(wb, t1.y, fmaf(wa, t0.y, acc.y));
-                acc.z = fmaf(wb, t1.z, fmaf(wa, t0.z, acc.z));
-                acc.w = fmaf(wb, t1.w, fmaf(wa, t0.w, acc.w));
-            }
+        for (int k = 0; k < 4; ++k) {  // the rows (y, z) of the taps
+            const float wyz = ((k & 1) ? f[1] : 1.0f - f[1]) * ((k >> 1) ? f[2] : 1.0f - f[2]);
+            const float4 t0 = tf_classify(tf, v[2 * k]), t1 = tf_classify(tf, v[2 * k + 1]);
+            const float wa = (1.0f - f[0]) * wyz, wb = f[0] * wyz;
+            acc.x = fmaf(wb, t1.x, fmaf(wa, t0.x, acc.x));
+            acc.y = fmaf(wb, t1.y, fmaf(wa, t0.y, acc.y));
+            acc.z = fmaf(wb, t1.z, fmaf(wa, t0.z, acc.z));
+            acc.w = fmaf(wb, t1.w, fmaf(wa, t0.w, acc.w));
         }
         return acc;
     }
@@ -498,10 +683,12 @@ __device__ __forceinline__ int quick_skip(const BrickView &bv, const uint8_t *__
 }
 
 // Launchers (return cudaSuccess or the launch error).
-cudaError_t launch_pad_volume(const void *src, int dtype, const int n[3], void *dst, int pnx,
-                              int pny, int pnz, cudaStream_t st);
-cudaError_t launch_replicate_x4(const void *src, int dtype, const int n[3], float4 *dst,
-                                cudaStream_t st);
+// Writes a volume's resident copies: the padded one (VolView) and the render layout (rep_view
+// gives its extents; rep_bytes its size).
+ReplView rep_view(const void *base, int dtype, const int n[3]);
+size_t rep_bytes(int dtype, const int n[3]);
+cudaError_t launch_volume_layouts(const void *src, int dtype, const int n[3], void *pad, int pnx,
+                                  void *rep, cudaStream_t st);
 cudaError_t launch_brick_minmax(const VolView &v, int B, void *mn, void *mx, cudaStream_t st);
 cudaError_t launch_occupancy(const void *mn, const void *mx, int dtype, long nbricks,
                              const int *prefix_dev, float lo, float du, uint8_t *occ,
