@@ -63,8 +63,8 @@ __device__ __forceinline__ void eval_sample(const RenderLaunch &L, const int ip[
     floor_small(u, i0);
     e.i0 = min(i0, 254);
     e.fu = u - (float)e.i0;
-    const float4 c0 = __ldg(L.tf.rgba + e.i0);
-    e.drgba = __ldg(L.tf.drgba + e.i0);
+    const float4 c0 = __ldg(L.tf.tab + 2 * e.i0);
+    e.drgba = __ldg(L.tf.tab + 2 * e.i0 + 1);
     e.rgba.x = fmaf(e.fu, e.drgba.x, c0.x);
     e.rgba.y = fmaf(e.fu, e.drgba.y, c0.y);
     e.rgba.z = fmaf(e.fu, e.drgba.z, c0.z);
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS) adjoint_kernel(AdjointLaunch A
             floor_small(u, i0);
             i0 = min(i0, 254);
             const float fu = u - (float)i0;
-            const float4 c0 = __ldg(L.tf.rgba + i0), dc = __ldg(L.tf.drgba + i0);
+            const float4 c0 = __ldg(L.tf.tab + 2 * i0), dc = __ldg(L.tf.tab + 2 * i0 + 1);
             const float r = fmaf(fu, dc.x, c0.x), gg = fmaf(fu, dc.y, c0.y);
             const float b = fmaf(fu, dc.z, c0.z), araw = fmaf(fu, dc.w, c0.w);
             const float a = fminf(fmaxf(araw, 0.0f), ALPHA_MAX);

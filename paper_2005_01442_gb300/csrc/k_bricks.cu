@@ -14,79 +14,114 @@
 namespace vrc {
 
 // ------------------------------------------------------------------ volume layouts ------
-// One warp per row (y', z') of the padded copy: it writes that row and the row of render
-// entries (ReplView), reading the source rows through L1 (each source voxel comes from HBM
-// once). Consecutive lanes write consecutive entries; the entries stream past L2 (the padded
-// copy, which the brick table reads next, may stay).
-// Bound: HBM, 2 (or 4) bytes read, as many padded and 16 of render layout written per voxel.
-// 512^2 x 400 int16 (2.1 GB): 386 us against 817 us for one kernel per layout with 64-bit
-// divisions per element; 256^3 float32: 61 us against 151 us.
-constexpr int VL_WARPS = 8;
+// One warp per 2 x 2 rows (y', z') of the padded copy: it writes those rows and the row of blocks
+// of render entries (ReplView) at the same place. The 3 x 3 rows it needs go through shared
+// memory, VL_SPAN words of each at a time (each source voxel comes from HBM once, the rest from
+// L2), from where consecutive lanes write consecutive 32-byte pieces of the blocks, past L2 (the
+// padded copy, which the brick table reads next, may stay). Words of a row lie VL_Y and VL_Z
+// apart, so that the four rows read at once fall on different banks.
+// Bound: HBM, 2 (or 4) bytes read, as many padded and 16 (32) of render layout written per voxel.
+// 512^2 x 400 int16 (2.1 GB): 356 us, 5.9 TB/s; a warp per row that read its four source rows
+// element by element, which the L1 data path bound: 388 us. 256^3 float32 (0.67 GB): 119 us.
+constexpr int VL_WARPS = 8, VL_SPAN = 128, VL_Y = 136, VL_Z = 432;
+
+// 32 bytes to a 32-byte boundary, not kept in L2.
+__device__ __forceinline__ void store32_streaming(void *p, const uint32_t v[8]) {
+    asm volatile("st.global.cs.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]),
+                 "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
 
 template <typename T>
 __global__ void __launch_bounds__(32 * VL_WARPS)
     volume_layouts_kernel(const T *__restrict__ src, int nx, int ny, int nz, T *__restrict__ pad,
-                          int pnx, uint4 *__restrict__ rep, int rnx, int rny, int rnz) {
-    const int lane = threadIdx.x & 31;
-    const unsigned row = blockIdx.x * VL_WARPS + (threadIdx.x >> 5);
-    const unsigned pny = ny + 2 * PAD;
-    const int y = (int)(row % pny), z = (int)(row / pny);
-    if (z >= nz + 2 * PAD) return;
-    auto source = [&](int yy, int zz) {
-        return src + ((size_t)min(max(zz - PAD, 0), nz - 1) * ny + min(max(yy - PAD, 0), ny - 1)) *
-                         nx;
-    };
-    const T *s0 = source(y, z);
-    {  // padded row, 4 elements per lane (pnx is a multiple of 8)
-        T *out = pad + (size_t)row * pnx;
-        for (int x = 4 * lane; x < pnx; x += 128) {
-            T v[4];
+                          int pnx, char *__restrict__ rep, int rnx, int rny, int rnz) {
+    constexpr int PER = 4 / (int)sizeof(T), SPAN = VL_SPAN * PER;  // voxels a word, a span
+    constexpr int ENTRY = sizeof(T) == 2 ? 16 : 32;
+    __shared__ __align__(16) uint32_t s_rows[VL_WARPS][3 * VL_Z];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *rows = s_rows[warp];
+    const unsigned unit = blockIdx.x * VL_WARPS + warp;
+    const int pny = ny + 2 * PAD, pnz = nz + 2 * PAD;
+    const unsigned ny2 = (unsigned)(pny + 1) >> 1;
+    const int by = (int)(unit % ny2), bz = (int)(unit / ny2);
+    if (2 * bz >= pnz) return;
+    const T *from[9];  // source rows of the padded rows (2 by + r % 3, 2 bz + r / 3)
+    uintptr_t low = 0;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = s0[min(max(x + e - PAD, 0), nx - 1)];
-            if constexpr (sizeof(T) == 2) memcpy(out + x, v, 8);
-            else *(float4 *)(out + x) = make_float4(v[0], v[1], v[2], v[3]);
-        }
+    for (int r = 0; r < 9; ++r) {
+        from[r] = src + ((size_t)min(max(2 * bz + r / 3 - PAD, 0), nz - 1) * ny +
+                         min(max(2 * by + r % 3 - PAD, 0), ny - 1)) * nx;
+        low |= (uintptr_t)from[r];
     }
-    if (y >= rny || z >= rnz) return;
-    uint4 *out = rep + ((size_t)z * rny + y) * rnx;
-    if constexpr (sizeof(T) == 2) {
-        const T *s1 = source(y + 1, z), *s2 = source(y, z + 1), *s3 = source(y + 1, z + 1);
-        const int half = rnx >> 1;
-        // int16: bias 32768, i.e. the sign bit flipped
-        const uint32_t flip = (T)-1 < (T)0 ? 0x80008000u : 0u;
-        // lane k: the entries x' = 2k and 2k + 1, i.e. voxels 2k-2 .. 2k of the four rows, the
-        // first two in one load where they lie inside an even-aligned row
-        const bool words = ((uintptr_t)s0 & 3) == 0 && ((uintptr_t)s1 & 3) == 0 &&
-                           ((uintptr_t)s2 & 3) == 0 && ((uintptr_t)s3 & 3) == 0;
-        for (int k = lane; k < half; k += 32) {
-            const T *rows[4] = {s0, s1, s2, s3};
-            const int x0 = 2 * k - 2, xc = min(2 * k, nx - 1);
-            uint32_t a[4], c[4];  // (voxel 2k-2, 2k-1), voxel 2k
-            if (words && x0 >= 0 && x0 + 1 < nx) {
+    const bool words = (low & 3) == 0;  // 16-bit voxels 2i, 2i + 1 in one load
+    const bool blocks = by < rny && bz < rnz;
+    char *out = rep + ((size_t)bz * rny + by) * rnx * 8 * ENTRY;
+    for (int x0 = 0; x0 < max(pnx, 2 * rnx); x0 += SPAN) {
+        __syncwarp();  // the span before has been read
+        // padded elements x0 .. x0 + SPAN + 3
+        for (int i = lane; i < VL_SPAN + 4 / PER; i += 32) {
+            const int x = x0 + i * PER - PAD;
+            uint32_t w[9];
+            if (sizeof(T) == 4 || (words && x >= 0 && x + 1 < nx)) {
+                const int xc = sizeof(T) == 4 ? min(max(x, 0), nx - 1) : x;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) a[r] = *(const uint32_t *)(rows[r] + x0);
+                for (int r = 0; r < 9; ++r) w[r] = *(const uint32_t *)(from[r] + xc);
             } else {
-                const int xa = min(max(x0, 0), nx - 1), xb = min(max(x0 + 1, 0), nx - 1);
+                const int xa = min(max(x, 0), nx - 1), xb = min(max(x + 1, 0), nx - 1);
 #pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    a[r] = (uint32_t)(uint16_t)rows[r][xa] | (uint32_t)(uint16_t)rows[r][xb] << 16;
+                for (int r = 0; r < 9; ++r)
+                    w[r] = (uint32_t)(uint16_t)from[r][xa] | (uint32_t)(uint16_t)from[r][xb] << 16;
             }
 #pragma unroll
-            for (int r = 0; r < 4; ++r) c[r] = (uint16_t)rows[r][xc];
-            // words (x, y): lower z in the low half; rows 0, 1: y, y+1 at z; 2, 3: at z+1
-            auto lo = [&](uint32_t u, uint32_t v) { return __byte_perm(u, v, 0x5410) ^ flip; };
-            auto hi = [&](uint32_t u, uint32_t v) { return __byte_perm(u, v, 0x7632) ^ flip; };
-            __stcs(out + k, make_uint4(lo(a[0], a[2]), hi(a[0], a[2]), lo(a[1], a[3]),
-                                       hi(a[1], a[3])));
-            __stcs(out + half + k, make_uint4(hi(a[0], a[2]), lo(c[0], c[2]), hi(a[1], a[3]),
-                                              lo(c[1], c[3])));
+            for (int r = 0; r < 9; ++r) rows[(r % 3) * VL_Y + (r / 3) * VL_Z + i] = w[r];
         }
-    } else {
-        for (int x = lane; x < rnx; x += 32) {
-            float v[4];
+        __syncwarp();
 #pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = s0[min(max(x + e - PAD, 0), nx - 1)];
-            __stcs((float4 *)out + x, make_float4(v[0], v[1], v[2], v[3]));
+        for (int r = 0; r < 4; ++r) {  // padded rows, 4 elements per lane (pnx is a multiple of 8)
+            const int y = 2 * by + (r & 1), z = 2 * bz + (r >> 1);
+            const uint32_t *s0 = rows + (r & 1) * VL_Y + (r >> 1) * VL_Z;
+            if (y >= pny || z >= pnz) continue;
+            T *to = pad + ((size_t)z * pny + y) * pnx;
+            for (int x = x0 + 4 * lane; x < min(pnx, x0 + SPAN); x += 128) {
+                if constexpr (sizeof(T) == 2)
+                    *(uint2 *)(to + x) = *(const uint2 *)(s0 + (x - x0) / 2);
+                else *(uint4 *)(to + x) = *(const uint4 *)(s0 + (x - x0));
+            }
+        }
+        if (!blocks) continue;
+        const int kend = min(rnx - x0 / 2, SPAN / 2);
+        if constexpr (sizeof(T) == 2) {
+            // lane: the entries x' = 2k, 2k + 1 of (y', z') = (2 by + g, 2 bz + h) in block k
+            const int g = lane & 1, h = (lane >> 1) & 1;
+            const uint32_t *s0 = rows + g * VL_Y + h * VL_Z;
+            // int16: bias 32768, i.e. the sign bit flipped
+            const uint32_t flip = (T)-1 < (T)0 ? 0x80008000u : 0u;
+            char *to = out + (size_t)(x0 / 2) * 8 * ENTRY + 32 * (lane & 3);
+            for (int k = lane >> 2; k < kend; k += 8) {
+                uint32_t e[3][2];  // pairs of voxel 2k - 2 + i of row y
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const uint32_t *a = s0 + y * VL_Y + k, *b = a + VL_Z;
+                    e[0][y] = __byte_perm(a[0], b[0], 0x5410) ^ flip;
+                    e[1][y] = __byte_perm(a[0], b[0], 0x7632) ^ flip;
+                    e[2][y] = __byte_perm(a[1], b[1], 0x5410) ^ flip;
+                }
+                const uint32_t v[8] = {e[0][0], e[1][0], e[0][1], e[1][1],
+                                       e[1][0], e[2][0], e[1][1], e[2][1]};
+                store32_streaming(to + k * (8 * ENTRY), v);
+            }
+        } else {
+            // lane: the entry of slot lane & 7 in block k
+            const int g = (lane >> 1) & 1, h = (lane >> 2) & 1;
+            const uint32_t *s0 = rows + g * VL_Y + h * VL_Z + (lane & 1);
+            char *to = out + (size_t)(x0 / 2) * 8 * ENTRY + ENTRY * (lane & 7);
+            for (int k = lane >> 3; k < kend; k += 4) {
+                const uint32_t *a = s0 + 2 * k, *b = a + VL_Z;
+                const uint32_t v[8] = {a[0], b[0], a[1], b[1],
+                                       a[VL_Y], b[VL_Y], a[VL_Y + 1], b[VL_Y + 1]};
+                store32_streaming(to + k * (8 * ENTRY), v);
+            }
         }
     }
 }
@@ -94,38 +129,40 @@ __global__ void __launch_bounds__(32 * VL_WARPS)
 ReplView rep_view(const void *base, int dtype, const int n[3]) {
     ReplView r;
     r.base = base;
-    r.half = dtype == DT_F32 ? 0 : (n[0] + 4) / 2;
-    r.rnx = dtype == DT_F32 ? n[0] + 1 : 2 * r.half;
-    r.rny = n[1] + (dtype == DT_F32 ? 4 : 3);
+    r.packed = dtype != DT_F32;
+    r.rnx = (n[0] + 4) / 2;
+    r.rny = (n[1] + 4) / 2;
+    r.row = (r.packed ? 128 : 256) * (size_t)r.rnx;
+    r.slice = r.row * r.rny;
     r.magic = 8388608.0f + (dtype == DT_I16 ? 32768.0f : 0.0f);
     return r;
 }
 
 size_t rep_bytes(int dtype, const int n[3]) {
     const ReplView r = rep_view(nullptr, dtype, n);
-    return 16 * (size_t)r.rnx * r.rny * (n[2] + (dtype == DT_F32 ? 4 : 3));
+    return r.slice * ((n[2] + 4) / 2);
 }
 
 cudaError_t launch_volume_layouts(const void *src, int dtype, const int n[3], void *pad, int pnx,
                                   void *rep, cudaStream_t st) {
     const ReplView r = rep_view(rep, dtype, n);
-    const int rnz = n[2] + (dtype == DT_F32 ? 4 : 3);
-    const long rows = (long)(n[1] + 2 * PAD) * (n[2] + 2 * PAD);
-    const unsigned blocks = (unsigned)((rows + VL_WARPS - 1) / VL_WARPS);
+    const int rnz = (n[2] + 4) / 2;
+    const long units = (long)((n[1] + 2 * PAD + 1) / 2) * ((n[2] + 2 * PAD + 1) / 2);
+    const unsigned blocks = (unsigned)((units + VL_WARPS - 1) / VL_WARPS);
     switch (dtype) {
     case DT_U16:
         volume_layouts_kernel<uint16_t><<<blocks, 32 * VL_WARPS, 0, st>>>(
-            (const uint16_t *)src, n[0], n[1], n[2], (uint16_t *)pad, pnx, (uint4 *)rep, r.rnx,
+            (const uint16_t *)src, n[0], n[1], n[2], (uint16_t *)pad, pnx, (char *)rep, r.rnx,
             r.rny, rnz);
         break;
     case DT_I16:
         volume_layouts_kernel<int16_t><<<blocks, 32 * VL_WARPS, 0, st>>>(
-            (const int16_t *)src, n[0], n[1], n[2], (int16_t *)pad, pnx, (uint4 *)rep, r.rnx,
+            (const int16_t *)src, n[0], n[1], n[2], (int16_t *)pad, pnx, (char *)rep, r.rnx,
             r.rny, rnz);
         break;
     default:
         volume_layouts_kernel<float><<<blocks, 32 * VL_WARPS, 0, st>>>(
-            (const float *)src, n[0], n[1], n[2], (float *)pad, pnx, (uint4 *)rep, r.rnx, r.rny,
+            (const float *)src, n[0], n[1], n[2], (float *)pad, pnx, (char *)rep, r.rnx, r.rny,
             rnz);
     }
     return cudaGetLastError();
@@ -556,7 +593,7 @@ cudaError_t launch_cellmask_rows(const uint32_t *cells, const int n[3], uint32_t
 // from i (front sample) to k (back sample) by PREINT_K equal sub-steps (midpoint rule, each
 // with the opacity correction alpha = 1 - (1 - a)^(ds / PREINT_K)); (associated rgb, opacity).
 // Computed in double (65536 entries, 32 sub-steps: negligible), stored as float4.
-__global__ void preint_table_kernel(const float4 *__restrict__ rgba, float ds,
+__global__ void preint_table_kernel(const float4 *__restrict__ tf_tab, float ds,
                                     float4 *__restrict__ tab) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= 256 * 256) return;
@@ -568,7 +605,7 @@ __global__ void preint_table_kernel(const float4 *__restrict__ rgba, float ds,
         int i0 = (int)floor(u);
         i0 = i0 > 254 ? 254 : i0;
         const double f = u - i0;
-        const float4 a = rgba[i0], b = rgba[i0 + 1];
+        const float4 a = tf_tab[2 * i0], b = tf_tab[2 * i0 + 2];
         const double r = (1.0 - f) * a.x + f * b.x, g = (1.0 - f) * a.y + f * b.y;
         const double bl = (1.0 - f) * a.z + f * b.z;
         double al = (1.0 - f) * a.w + f * b.w;
@@ -582,8 +619,8 @@ __global__ void preint_table_kernel(const float4 *__restrict__ rgba, float ds,
     tab[e] = make_float4((float)c0, (float)c1, (float)c2, (float)(1.0 - T));
 }
 
-cudaError_t launch_preint_table(const float4 *rgba, float ds, float4 *tab, cudaStream_t st) {
-    preint_table_kernel<<<256, 256, 0, st>>>(rgba, ds, tab);
+cudaError_t launch_preint_table(const float4 *tf_tab, float ds, float4 *tab, cudaStream_t st) {
+    preint_table_kernel<<<256, 256, 0, st>>>(tf_tab, ds, tab);
     return cudaGetLastError();
 }
 

@@ -55,17 +55,23 @@ __device__ __forceinline__ int advance_to_occupied(const RayPos &rp, const Rende
 // before the first block with a composited sample in each segment (-1 for segments without
 // one), every segment from the first to the last such one (written by the group's lanes in
 // turn), and the last composited sample.
-template <bool ESL, int G, int MODE = MODE_CUBIC_POST, bool CKPT = false>
+//
+// PACKED: the volume's render layout where the kernel is compiled for one (1: 16-bit voxels, 0:
+// float32), -1 where it takes either. Pf and inv_df are read at leaps only and may lie in shared
+// memory.
+template <bool ESL, int G, int MODE = MODE_CUBIC_POST, bool CKPT = false, int PACKED = -1>
 __device__ __forceinline__ void group_march(const RenderLaunch &L, const RayPos &rp,
                                             const uint8_t *__restrict__ dist, const float Pf[3],
                                             const float df[3], const float inv_df[3],
                                             float inv_step, int jlo, unsigned gmask, int q,
                                             int gbase, float &RC0, float &RC1, float &RC2,
-                                            float &RT, unsigned long long &executed,
+                                            float &RT, unsigned &executed,
                                             unsigned &resampled, CkState *ck = nullptr) {
     constexpr int SH = G == 32 ? 5 : G == 16 ? 4 : G == 8 ? 3 : 2;
     constexpr unsigned low = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     const float step = L.grid.step, thr = L.grid.ert;
+    ReplView rep = L.rep;
+    if (PACKED >= 0) rep.packed = PACKED;
     int blk = jlo >> SH;
     int cache_lin = -1;     // brick of this lane's last sample
     bool cache_occ = false;
@@ -89,7 +95,7 @@ __device__ __forceinline__ void group_march(const RenderLaunch &L, const RayPos 
                 live = in_occ && (!L.cells || cell_open(L.cells, L.grid.n, ip));
             }
             if (live) {
-                const float4 rgba = sample_rgba<MODE>(L.rep, L.tf, ip, f, df, &L.phong);
+                const float4 rgba = sample_rgba<MODE>(rep, L.tf, ip, f, df, &L.phong);
                 const float alpha = segment_alpha(rgba.w, delta);
                 e0 = alpha * rgba.x;
                 e1 = alpha * rgba.y;

@@ -30,9 +30,9 @@ __global__ void __launch_bounds__(32 * SPLIT_RAY_WARPS, 16 / SPLIT_RAY_WARPS)
 // Four CTAs per SM (64 registers, a few spills): the march is bound by the latency of
 // dependent loads, and 32 resident warps hide it better than 24 at 80 registers (measured:
 // 0.377 vs 0.392 ms per 1024^2 CT frame; five CTAs at 48 registers spill too much).
-template <bool ESL, int MODE, bool CKPT = false>
+template <bool ESL, int MODE, bool CKPT, int PACKED>
 __global__ void __launch_bounds__(32 * SPLIT_WARPS, 4) split_tail_kernel(RenderLaunch L) {
-    split_tail_body<ESL, MODE, CKPT>(L);
+    split_tail_body<ESL, MODE, CKPT, PACKED>(L);
 }
 
 namespace {
@@ -46,7 +46,7 @@ int tail_ctas(cudaError_t &e) {
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, split_tail_kernel<true, MODE_CUBIC_POST>, 32 * SPLIT_WARPS, 0);
+        &per_sm, split_tail_kernel<true, MODE_CUBIC_POST, false, 1>, 32 * SPLIT_WARPS, 0);
     if (e != cudaSuccess) return 0;
     const int n = sms * (per_sm > 0 ? per_sm : 1);
     if (dev >= 0 && dev < 64) cached[dev] = n;
@@ -54,10 +54,15 @@ int tail_ctas(cudaError_t &e) {
 }
 }  // namespace
 
+template <int MODE, bool CKPT, int PACKED>
+static void launch_tail_of(const RenderLaunch &L, int ctas, cudaStream_t st) {
+    if (L.dist) split_tail_kernel<true, MODE, CKPT, PACKED><<<ctas, 32 * SPLIT_WARPS, 0, st>>>(L);
+    else split_tail_kernel<false, MODE, CKPT, PACKED><<<ctas, 32 * SPLIT_WARPS, 0, st>>>(L);
+}
 template <int MODE, bool CKPT = false>
 static void launch_tail(const RenderLaunch &L, int ctas, cudaStream_t st) {
-    if (L.dist) split_tail_kernel<true, MODE, CKPT><<<ctas, 32 * SPLIT_WARPS, 0, st>>>(L);
-    else split_tail_kernel<false, MODE, CKPT><<<ctas, 32 * SPLIT_WARPS, 0, st>>>(L);
+    if (L.rep.packed) launch_tail_of<MODE, CKPT, 1>(L, ctas, st);
+    else launch_tail_of<MODE, CKPT, 0>(L, ctas, st);
 }
 
 cudaError_t launch_render_split(const RenderLaunch &L, cudaStream_t st) {

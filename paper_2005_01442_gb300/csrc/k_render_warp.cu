@@ -85,8 +85,10 @@ __global__ void __launch_bounds__(WC_RAYS, 2) render_warp_kernel(RenderLaunch L)
         const uint8_t *dist = nullptr;
         if (ESL) dist = L.dist + octant_of(df) * nbricks;
         float RC0 = 0.0f, RC1 = 0.0f, RC2 = 0.0f, RT = 1.0f;
+        unsigned ex = 0;
         group_march<ESL, G>(L, rp, dist, Pf, df, inv_df, inv_step, s_rec[qi].j0, gmask, q, gbase,
-                            RC0, RC1, RC2, RT, executed, resampled);
+                            RC0, RC1, RC2, RT, ex, resampled);
+        executed += ex;
         if (q == 0) L.out[pix] = make_float4(RC0, RC1, RC2, 1.0f - RT);
     }
 

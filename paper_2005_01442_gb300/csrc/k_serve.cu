@@ -100,8 +100,7 @@ __device__ __forceinline__ void serve_rays_body(const RenderLaunch &L, unsigned 
     const unsigned gmask = ((1u << SPLIT_G) - 1u) << gbase;
     const float inv_step = 1.0f / L.grid.step;
     const long nbricks = ESL ? (long)L.bricks.nb[0] * L.bricks.nb[1] * L.bricks.nb[2] : 0;
-    unsigned long long executed = 0;
-    unsigned resampled = 0;
+    unsigned executed = 0, resampled = 0;
     for (unsigned c = c0 + group; c < c0 + chunk; c += 2) {
         const unsigned qi = c < nf ? c : L.split.cap - 1u - (c - nf);
         RayPos rp;

@@ -51,12 +51,16 @@ struct Volume {
     std::map<long, Occ> occ;        // key: tf_id * 2 + (B == 16)
 };
 
+// What a transfer function keeps on the device, uploaded in one copy.
+struct TfTables {
+    float4 tab[512];    // entry k and the difference to entry k + 1 (TfView)
+    int prefix[257];    // non-zero opacities before entry k
+    uint8_t zrun[256];  // run id of each zero-opacity entry (0: non-zero entry)
+};
+
 struct Tf {
     float lo = 0, hi = 1, du = 255;
-    float4 *rgba = nullptr;   // 256
-    float4 *drgba = nullptr;  // 256
-    int *prefix = nullptr;    // 257
-    uint8_t *zrun = nullptr;  // 256: run id of each zero-opacity entry (0: non-zero entry)
+    TfTables *dev = nullptr;
     unsigned version = 0;
     float4 *preint = nullptr;    // 256 x 256 pre-integration table, built on first use
     float preint_step = -1.0f;   // the step it was built for
@@ -183,10 +187,7 @@ void free_volume(Volume &v) {
 }
 
 void free_tf(Tf &t) {
-    cudaFree(t.rgba);
-    cudaFree(t.drgba);
-    cudaFree(t.prefix);
-    cudaFree(t.zrun);
+    cudaFree(t.dev);
     cudaFree(t.preint);
 }
 
@@ -313,35 +314,26 @@ vrc_status upload_tf(vrc_ctx *ctx, Tf &t, const float *rgba, float lo, float hi)
         return fail(ctx, VRC_ERR_ARG, "transfer function window needs finite hi > lo");
     for (int i = 0; i < 1024; ++i)
         if (!isfinite(rgba[i])) return fail(ctx, VRC_ERR_ARG, "transfer function has non-finite entries");
-    std::vector<float4> a(256), d(256);
-    std::vector<int> pre(257);
-    std::vector<uint8_t> zrun(256);
-    pre[0] = 0;
+    TfTables h;
+    h.prefix[0] = 0;
     int runs = 0;
     for (int i = 0; i < 256; ++i) {
-        a[i] = make_float4(rgba[4 * i], rgba[4 * i + 1], rgba[4 * i + 2], rgba[4 * i + 3]);
-        const bool nz = rgba[4 * i + 3] > 0.0f;
-        pre[i + 1] = pre[i] + (nz ? 1 : 0);
+        const float *c = rgba + 4 * i, *n = c + 4;
+        h.tab[2 * i] = make_float4(c[0], c[1], c[2], c[3]);
+        h.tab[2 * i + 1] = i < 255 ? make_float4(n[0] - c[0], n[1] - c[1], n[2] - c[2], n[3] - c[3])
+                                   : make_float4(0, 0, 0, 0);
+        const bool nz = c[3] > 0.0f;
+        h.prefix[i + 1] = h.prefix[i] + (nz ? 1 : 0);
         if (!nz && (i == 0 || rgba[4 * i - 1] > 0.0f)) ++runs;  // at most 128 runs
-        zrun[i] = nz ? 0 : (uint8_t)runs;
+        h.zrun[i] = nz ? 0 : (uint8_t)runs;
     }
-    for (int i = 0; i < 255; ++i)
-        d[i] = make_float4(rgba[4 * i + 4] - rgba[4 * i], rgba[4 * i + 5] - rgba[4 * i + 1],
-                           rgba[4 * i + 6] - rgba[4 * i + 2], rgba[4 * i + 7] - rgba[4 * i + 3]);
-    d[255] = make_float4(0, 0, 0, 0);
-    if (!t.rgba) {
-        CK(cudaMalloc(&t.rgba, 256 * sizeof(float4)), "cudaMalloc(tf)");
-        CK(cudaMalloc(&t.drgba, 256 * sizeof(float4)), "cudaMalloc(tf)");
-        CK(cudaMalloc(&t.prefix, 257 * sizeof(int)), "cudaMalloc(tf)");
-        CK(cudaMalloc(&t.zrun, 256), "cudaMalloc(tf)");
+    if (!t.dev) {
+        CK(cudaMalloc(&t.dev, sizeof(TfTables)), "cudaMalloc(tf)");
     } else {
         // tables may be in use by queued kernels on any stream
         CK(cudaDeviceSynchronize(), "cudaDeviceSynchronize(tf update)");
     }
-    CK(cudaMemcpy(t.rgba, a.data(), 256 * sizeof(float4), cudaMemcpyHostToDevice), "tf upload");
-    CK(cudaMemcpy(t.drgba, d.data(), 256 * sizeof(float4), cudaMemcpyHostToDevice), "tf upload");
-    CK(cudaMemcpy(t.prefix, pre.data(), 257 * sizeof(int), cudaMemcpyHostToDevice), "tf upload");
-    CK(cudaMemcpy(t.zrun, zrun.data(), 256, cudaMemcpyHostToDevice), "tf upload");
+    CK(cudaMemcpy(t.dev, &h, sizeof(h), cudaMemcpyHostToDevice), "tf upload");
     volatile float range = hi - lo;
     t.lo = lo;
     t.hi = hi;
@@ -378,10 +370,10 @@ vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStre
         o.brick_version = o.tf_version = 0;
     }
     if (o.brick_version != b.version || o.tf_version != t.version) {
-        CK(launch_occupancy(b.mn, b.mx, v.dtype, b.count(), t.prefix, t.lo, t.du, o.dev, st),
+        CK(launch_occupancy(b.mn, b.mx, v.dtype, b.count(), t.dev->prefix, t.lo, t.du, o.dev, st),
            "occupancy launch");
         CK(launch_box_dist(o.dev, b.nb, o.scratch, o.dist, st), "distance launch");
-        CK(launch_cellmask(view_of(v), B, b.nb, o.dev, t.zrun, t.lo, t.du, o.cells, st),
+        CK(launch_cellmask(view_of(v), B, b.nb, o.dev, t.dev->zrun, t.lo, t.du, o.cells, st),
            "cell mask launch");
         o.brick_version = b.version;
         o.tf_version = t.version;
@@ -512,8 +504,7 @@ vrc_status box_rect(vrc_ctx *ctx, const vrc_camera *cam, const float lo[3], cons
 
 TfView tf_view(const Tf &t) {
     TfView tv;
-    tv.rgba = t.rgba;
-    tv.drgba = t.drgba;
+    tv.tab = t.dev->tab;
     tv.lo = t.lo;
     tv.hi = t.hi;
     tv.du = t.du;
@@ -567,7 +558,7 @@ vrc_status prepare_render(vrc_ctx *ctx, int vol_id, int tf_id, const vrc_camera 
     if (p->preint) {
         if (!t->preint) CK(cudaMalloc(&t->preint, 256 * 256 * sizeof(float4)), "cudaMalloc(preint)");
         if (t->preint_step != p->step || t->preint_version != t->version) {
-            CK(launch_preint_table(t->rgba, p->step, t->preint, st), "pre-integration launch");
+            CK(launch_preint_table(t->dev->tab, p->step, t->preint, st), "pre-integration launch");
             t->preint_step = p->step;
             t->preint_version = t->version;
         }
@@ -1354,13 +1345,13 @@ extern "C" vrc_status vrc_render_noalloc(vrc_ctx *ctx, int vol_id, int tf_id,
         uint8_t *dist = scratch + dist_off;
         int *svt = (int *)(scratch + svt_off);
         // every byte these kernels read is written first by this call: nothing to clear
-        CK(launch_occupancy(b->mn, b->mx, v->dtype, b->count(), t->prefix, t->lo, t->du, occ, st),
+        CK(launch_occupancy(b->mn, b->mx, v->dtype, b->count(), t->dev->prefix, t->lo, t->du, occ, st),
            "occupancy launch");
         CK(launch_box_dist(occ, b->nb, svt, dist, st), "distance launch");
         // the cell mask too when it fits behind the tables (it only saves work)
         if (cells_off + cellmask_bytes(v->n) <= (size_t)VRC_NOALLOC_SCRATCH_BYTES) {
             uint32_t *cells = (uint32_t *)(scratch + cells_off);
-            CK(launch_cellmask(view_of(*v), B, b->nb, occ, t->zrun, t->lo, t->du, cells, st),
+            CK(launch_cellmask(view_of(*v), B, b->nb, occ, t->dev->zrun, t->lo, t->du, cells, st),
                "cell mask launch");
             L.cells = cells;
         }

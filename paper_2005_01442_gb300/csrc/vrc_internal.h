@@ -28,28 +28,31 @@ struct VolView {
     int pnx, pny, pnz;
 };
 
-// The render layout of a resident volume: 16-byte entries, each voxel in several of them, so
-// that a sample reads its 64 taps with few aligned 16-byte loads. Indices are clamped to the
-// volume (clamp-to-edge) when the layout is written.
+// The render layout of a resident volume: each voxel in several entries, so that a sample reads
+// its 64 taps with few aligned wide loads. Entry (x', y', z') holds the 2^3 voxels from (x'-2,
+// y'-2, z'-2), x' in [0, nx+2] and so on, indices clamped to the volume (clamp-to-edge) when
+// the layout is written. A sample at base i reads the 8 entries (i0+1 + {0, 2}, i1+1 + {0, 2},
+// i2+1 + {0, 2}). The voxels lie in pairs along z, one pair per (x, y) with x fastest, as the
+// packed float32 arithmetic of the resampling takes them.
 //
-// float32: entry (x', y', z') holds the voxels x'-2 .. x'+1 of row (y'-2, z'-2); x' in [0, nx],
-//   y' in [0, ny+3], z' in [0, nz+3]. A sample at base i reads entries (i0+1, i1+1+b, i2+1+c),
-//   16 loads.
-// 16-bit: entry (x', y', z') holds the 2^3 voxels from (x'-2, y'-2, z'-2): four words, one per
-//   (x, y) with x fastest, low half the lower z, each voxel plus `bias` as an unsigned 16-bit
-//   value; x' in [0, nx+2] and so on. Along x the entries of even x' come first, then those of
-//   odd x' (`half` of each per row), since a sample reads entries of one parity: (i0+1 + {0, 2},
-//   i1+1 + {0, 2}, i2+1 + {0, 2}), 8 loads, pairs of them adjacent.
-//   Half the loads and bytes of the same volume as float4 rows: a dense 1024^2 frame of a 512^2
-//   x 400 CT was bound by the L1 data path (93% of its peak, 934 M wavefronts) and takes 2.79 ms
-//   (706 M) instead of 3.15; unpacking costs 96 instructions a sample, of which packed float32
-//   arithmetic saves 40 again. Float32 volumes keep the rows of 4: packing them by z would save
-//   the 40 but no load.
+// 16-bit: 16 bytes, a pair one word (low half the lower z), each voxel plus `bias` as an
+//   unsigned 16-bit value.
+// float32: 32 bytes.
+//
+// Entries lie in blocks of 2^3 (slot 4 (z' & 1) + 2 (y' & 1) + (x' & 1)), blocks in rows along x.
+// The render is bound by the L1 data path, which serves a line at a time: the samples of a warp
+// lie along rays, and a ray crosses fewer blocks than rows of entries.
+// Second phase of a dense 1024^2 frame of a 512^2 x 400 int16 CT, 105 M samples: 2.50 ms and 637
+// M wavefronts of the L1 data path in rows of entries, 2.36 ms and 563 M in blocks, 2.11 ms and
+// 481 M (72% of its rate; 75% of the issue slots) with table lookups of 32 bytes and a kernel per
+// voxel type as well. 256^3 float32 (17 M samples): 0.61 ms and 168 M with 16 loads of four
+// voxels along x in half the memory, 0.53 ms and 125 M so.
 struct ReplView {
     const void *base;
-    int rnx, rny;   // entries per row, rows per slice
-    int half;       // 16-bit: entries of each parity per row; 0: float32
-    float magic;    // 16-bit: 2^23 + bias
+    size_t row, slice;  // bytes from a block to the next along y and z
+    int rnx, rny;       // blocks per row, rows of blocks per slice
+    int packed;         // 16-bit voxels
+    float magic;        // 16-bit: 2^23 + bias
 };
 
 // Brick table of size B (min/max arrays of the voxel dtype, ceil(n/B) per axis).
@@ -60,10 +63,10 @@ struct BrickView {
     float margin;  // leap and quick-skip margin in voxels (leap_margin)
 };
 
-// Device transfer function: rgba[k] and the forward difference rgba[k+1] - rgba[k].
+// Device transfer function: table entry k at tab[2k], the forward difference to entry k + 1 (0 for
+// the last) at tab[2k + 1], 256 of each; a lookup is one 32-byte load.
 struct TfView {
-    const float4 *rgba;   // 256 entries
-    const float4 *drgba;  // 256 entries, drgba[255] = 0
+    const float4 *tab;
     float lo, hi, du;     // du = 255 / (hi - lo) in float32
 };
 
@@ -171,126 +174,139 @@ __device__ __forceinline__ f32x2 voxels2(uint32_t w, f32x2 sub) {
                 sub);
 }
 
-// 16-bit layout: entry of voxels (x, y, z) .. + 1, x >= -2 and so on.
-__device__ __forceinline__ const uint4 *entry16(const ReplView &rp, int x, int y, int z) {
-    x += 2;
-    const unsigned i = ((unsigned)(z + 2) * rp.rny + (unsigned)(y + 2)) * rp.rnx +
-                       ((x & 1) ? rp.half : 0) + (x >> 1);
-    return (const uint4 *)rp.base + i;
+// Entry (x', y', z') = (x + 2, y + 2, z + 2): the one that starts at voxel (x, y, z). Two entries
+// on along an axis lies the same slot of the next block: 8 entries on along x, 8 rnx along y.
+__device__ __forceinline__ unsigned entry_index(const ReplView &rp, int x, int y, int z) {
+    const unsigned X = x + 2, Y = y + 2, Z = z + 2;
+    return (((Z >> 1) * rp.rny + (Y >> 1)) * rp.rnx + (X >> 1)) * 8u +
+           ((Z & 1) * 4u + (Y & 1) * 2u + (X & 1));
 }
 
-__device__ __forceinline__ const float4 *entry32(const ReplView &rp, int x, int y, int z) {
-    const unsigned i = ((unsigned)(z + 2) * rp.rny + (unsigned)(y + 2)) * rp.rnx +
-                       (unsigned)(x + 2);
-    return (const float4 *)rp.base + i;
+// 32 bytes from a 32-byte boundary, through the read-only path.
+__device__ __forceinline__ void load32(const void *p, f32x2 v[4]) {
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
+        : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
+        : "l"(p));
+}
+
+// An entry as it lies in memory.
+template <bool PACKED>
+struct Entry {
+    static constexpr size_t SIZE = 16;
+    uint4 w;
+    __device__ __forceinline__ void load(const char *p) { w = __ldg((const uint4 *)p); }
+    // pair (x, y) = (k & 1, k >> 1) as float32
+    __device__ __forceinline__ f32x2 pair(int k, f32x2 sub) const {
+        return voxels2(k == 0 ? w.x : k == 1 ? w.y : k == 2 ? w.z : w.w, sub);
+    }
+};
+template <>
+struct Entry<false> {
+    static constexpr size_t SIZE = 32;
+    f32x2 v[4];
+    __device__ __forceinline__ void load(const char *p) { load32(p, v); }
+    __device__ __forceinline__ f32x2 pair(int k, f32x2) const { return v[k]; }
+};
+
+// The first of a sample's 8 entries, and entry (x, y, z) of them.
+template <bool PACKED>
+__device__ __forceinline__ const char *first_entry(const ReplView &rp, const int ip[3]) {
+    return (const char *)rp.base +
+           Entry<PACKED>::SIZE * (size_t)entry_index(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+}
+template <bool PACKED>
+__device__ __forceinline__ const char *entry_at(const ReplView &rp, const char *p, int x, int y,
+                                                int z) {
+    if (z) p += rp.slice;
+    if (y) p += rp.row;
+    return x ? p + 8 * Entry<PACKED>::SIZE : p;
 }
 
 // Calls fn(c, b, v) for the 16 tap rows (y ip1-1+b, z ip2-1+c) of base ip, c outermost; v holds
 // the voxels ip0-1 .. ip0+2 of the row.
-template <class Fn>
-__device__ __forceinline__ void for_rows(const ReplView &rp, const int ip[3], Fn fn) {
-    if (rp.half) {
-        const f32x2 sub = pack2(-rp.magic, -rp.magic);
-        const uint4 *p = entry16(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
-        const unsigned row2 = 2u * rp.rnx, slice2 = row2 * rp.rny;
+template <bool PACKED, class Fn>
+__device__ __forceinline__ void for_rows_of(const ReplView &rp, const int ip[3], Fn fn) {
+    const f32x2 sub = pack2(-rp.magic, -rp.magic);
+    const char *p = first_entry<PACKED>(rp, ip);
 #pragma unroll
-        for (int zh = 0; zh < 2; ++zh) {
-            float4 v[2][4];  // rows of the lower and the upper z
+    for (int zh = 0; zh < 2; ++zh) {
+        float4 v[2][4];  // rows of the lower and the upper z
 #pragma unroll
-            for (int yh = 0; yh < 2; ++yh) {
-                const uint4 *e = p + (zh ? slice2 : 0u) + (yh ? row2 : 0u);
-                const uint4 a = __ldg(e), b = __ldg(e + 1);
-                const float2 a0 = unpack2(voxels2(a.x, sub)), a1 = unpack2(voxels2(a.y, sub));
-                const float2 a2 = unpack2(voxels2(a.z, sub)), a3 = unpack2(voxels2(a.w, sub));
-                const float2 b0 = unpack2(voxels2(b.x, sub)), b1 = unpack2(voxels2(b.y, sub));
-                const float2 b2 = unpack2(voxels2(b.z, sub)), b3 = unpack2(voxels2(b.w, sub));
-                v[0][2 * yh] = make_float4(a0.x, a1.x, b0.x, b1.x);
-                v[1][2 * yh] = make_float4(a0.y, a1.y, b0.y, b1.y);
-                v[0][2 * yh + 1] = make_float4(a2.x, a3.x, b2.x, b3.x);
-                v[1][2 * yh + 1] = make_float4(a2.y, a3.y, b2.y, b3.y);
+        for (int yh = 0; yh < 2; ++yh) {
+            Entry<PACKED> l, u;
+            l.load(entry_at<PACKED>(rp, p, 0, yh, zh));
+            u.load(entry_at<PACKED>(rp, p, 1, yh, zh));
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float2 a = unpack2(l.pair(2 * k, sub)), b = unpack2(l.pair(2 * k + 1, sub));
+                const float2 c = unpack2(u.pair(2 * k, sub)), d = unpack2(u.pair(2 * k + 1, sub));
+                v[0][2 * yh + k] = make_float4(a.x, b.x, c.x, d.x);
+                v[1][2 * yh + k] = make_float4(a.y, b.y, c.y, d.y);
             }
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) fn(2 * zh + h, b, v[h][b]);
         }
-    } else {
-        const float4 *p = entry32(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
-        const unsigned slice = (unsigned)rp.rnx * rp.rny;
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) fn(c, b, __ldg(p + c * slice + b * rp.rnx));
+            for (int b = 0; b < 4; ++b) fn(2 * zh + h, b, v[h][b]);
     }
 }
+template <class Fn>
+__device__ __forceinline__ void for_rows(const ReplView &rp, const int ip[3], Fn fn) {
+    if (rp.packed) for_rows_of<true>(rp, ip, fn);
+    else for_rows_of<false>(rp, ip, fn);
+}
 
-// Cubic B-spline sample at integer base ip (taps ip-1 .. ip+2) with fractions f. Both layouts
-// sum the same products in the same order: along x, then y, then z.
-__device__ __forceinline__ float tricubic_rep(const ReplView &rp, const int ip[3],
-                                              const float f[3]) {
+// Cubic B-spline sample at integer base ip (taps ip-1 .. ip+2) with fractions f: sums along x,
+// then y, then z, two z at a time.
+template <bool PACKED>
+__device__ __forceinline__ float tricubic_of(const ReplView &rp, const int ip[3],
+                                             const float f[3]) {
+    const f32x2 sub = pack2(-rp.magic, -rp.magic);
+    const char *p = first_entry<PACKED>(rp, ip);
+    Entry<PACKED> e[2][2][2];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+        e[k >> 2][(k >> 1) & 1][k & 1].load(
+            entry_at<PACKED>(rp, p, k & 1, (k >> 1) & 1, k >> 2));
     float wx[4], wy[4], wz[4];
     bspline_w(f[0], wx);
     bspline_w(f[1], wy);
     bspline_w(f[2], wz);
-    float s = 0.0f;
-    if (rp.half) {
-        // two z at a time
-        const f32x2 sub = pack2(-rp.magic, -rp.magic);
-        f32x2 wx2[4], wy2[4];
+    f32x2 wx2[4], wy2[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            wx2[k] = pack2(wx[k], wx[k]);
-            wy2[k] = pack2(wy[k], wy[k]);
-        }
-        const uint4 *p = entry16(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
-        const unsigned row2 = 2u * rp.rnx, slice2 = row2 * rp.rny;
-        uint4 e[2][2][2];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            e[k >> 2][(k >> 1) & 1][k & 1] =
-                __ldg(p + ((k & 4) ? slice2 : 0u) + ((k & 2) ? row2 : 0u) + (k & 1));
-#pragma unroll
-        for (int zh = 0; zh < 2; ++zh) {
-            f32x2 plane = 0ull;
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const uint4 l = e[zh][b >> 1][0], u = e[zh][b >> 1][1];
-                f32x2 r = mul2(wx2[0], voxels2((b & 1) ? l.z : l.x, sub));
-                r = fma2(wx2[1], voxels2((b & 1) ? l.w : l.y, sub), r);
-                r = fma2(wx2[2], voxels2((b & 1) ? u.z : u.x, sub), r);
-                r = fma2(wx2[3], voxels2((b & 1) ? u.w : u.y, sub), r);
-                plane = fma2(wy2[b], r, plane);
-            }
-            const float2 pl = unpack2(plane);
-            s = fmaf(wz[2 * zh], pl.x, s);
-            s = fmaf(wz[2 * zh + 1], pl.y, s);
-        }
-        return s;
+    for (int k = 0; k < 4; ++k) {
+        wx2[k] = pack2(wx[k], wx[k]);
+        wy2[k] = pack2(wy[k], wy[k]);
     }
-    const float4 *p0 = entry32(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
-    const unsigned slice = (unsigned)rp.rnx * rp.rny;
+    float s = 0.0f;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float4 *pc = p0 + c * slice;
-        float plane = 0.0f;
+    for (int zh = 0; zh < 2; ++zh) {
+        f32x2 plane = 0ull;
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
-            const float4 v = __ldg(pc + b * rp.rnx);
-            float r = wx[0] * v.x;
-            r = fmaf(wx[1], v.y, r);
-            r = fmaf(wx[2], v.z, r);
-            r = fmaf(wx[3], v.w, r);
-            plane = fmaf(wy[b], r, plane);
+            const Entry<PACKED> &l = e[zh][b >> 1][0], &u = e[zh][b >> 1][1];
+            const int k = 2 * (b & 1);
+            f32x2 r = mul2(wx2[0], l.pair(k, sub));
+            r = fma2(wx2[1], l.pair(k + 1, sub), r);
+            r = fma2(wx2[2], u.pair(k, sub), r);
+            r = fma2(wx2[3], u.pair(k + 1, sub), r);
+            plane = fma2(wy2[b], r, plane);
         }
-        s = fmaf(wz[c], plane, s);
+        const float2 pl = unpack2(plane);
+        s = fmaf(wz[2 * zh], pl.x, s);
+        s = fmaf(wz[2 * zh + 1], pl.y, s);
     }
     return s;
+}
+__device__ __forceinline__ float tricubic_rep(const ReplView &rp, const int ip[3],
+                                              const float f[3]) {
+    return rp.packed ? tricubic_of<true>(rp, ip, f) : tricubic_of<false>(rp, ip, f);
 }
 
 // Pre-integrated classification: 256 x 256 table of slab (associated rgb, opacity), front
 // entry major (preint_table_kernel); PREINT_K sub-steps per entry.
 constexpr int PREINT_K = 32;
-cudaError_t launch_preint_table(const float4 *rgba, float ds, float4 *tab, cudaStream_t st);
+cudaError_t launch_preint_table(const float4 *tf_tab, float ds, float4 *tab, cudaStream_t st);
 
 // Bilinear lookup at clamped table coordinates (uf, ub) in [0, 255].
 __device__ __forceinline__ float4 preint_lookup(const float4 *__restrict__ tab, float uf,
@@ -313,26 +329,22 @@ __device__ __forceinline__ float4 preint_lookup(const float4 *__restrict__ tab, 
 }
 
 // The 8 voxels ip .. ip+1 (clamped), x fastest, then y, then z.
+template <bool PACKED>
+__device__ __forceinline__ void taps8_of(const ReplView &rp, const int ip[3], float v[8]) {
+    const f32x2 sub = pack2(-rp.magic, -rp.magic);
+    Entry<PACKED> e;
+    e.load((const char *)rp.base +
+           Entry<PACKED>::SIZE * (size_t)entry_index(rp, ip[0], ip[1], ip[2]));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float2 z = unpack2(e.pair(k, sub));
+        v[k] = z.x;
+        v[k + 4] = z.y;
+    }
+}
 __device__ __forceinline__ void taps8(const ReplView &rp, const int ip[3], float v[8]) {
-    if (rp.half) {
-        const f32x2 sub = pack2(-rp.magic, -rp.magic);
-        const uint4 e = __ldg(entry16(rp, ip[0], ip[1], ip[2]));
-        const uint32_t w[4] = {e.x, e.y, e.z, e.w};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float2 z = unpack2(voxels2(w[k], sub));
-            v[k] = z.x;
-            v[k + 4] = z.y;
-        }
-        return;
-    }
-    const float4 *p = entry32(rp, ip[0] - 1, ip[1], ip[2]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {  // components y and z: voxels ip0 and ip0 + 1
-        const float4 r = __ldg(p + (k >> 1) * ((unsigned)rp.rnx * rp.rny) + (k & 1) * rp.rnx);
-        v[2 * k] = r.y;
-        v[2 * k + 1] = r.z;
-    }
+    if (rp.packed) taps8_of<true>(rp, ip, v);
+    else taps8_of<false>(rp, ip, v);
 }
 
 // Trilinear sample at integer base ip with fractions f.
@@ -348,15 +360,29 @@ __device__ __forceinline__ float trilinear_rep(const ReplView &rp, const int ip[
 }
 
 // Post-classification of value v: u = (v - lo) * du on [0, 255], linear between entries.
+struct Classified {
+    float u_raw, fu;  // index coordinate before clamping, weight of the upper entry
+    int i0;           // lower entry
+    float4 c, dc;     // interpolated entry, table difference at i0
+};
+__device__ __forceinline__ Classified classify(const TfView &tf, float v) {
+    Classified k;
+    k.u_raw = (v - tf.lo) * tf.du;
+    const float u = fminf(fmaxf(k.u_raw, 0.0f), 255.0f);
+    floor_small(u, k.i0);
+    k.i0 = min(k.i0, 254);
+    k.fu = u - (float)k.i0;
+    f32x2 e[4];
+    load32(tf.tab + 2 * k.i0, e);
+    const float2 dxy = unpack2(e[2]), dzw = unpack2(e[3]);
+    k.dc = make_float4(dxy.x, dxy.y, dzw.x, dzw.y);
+    const f32x2 fu2 = pack2(k.fu, k.fu);
+    const float2 xy = unpack2(fma2(fu2, e[2], e[0])), zw = unpack2(fma2(fu2, e[3], e[1]));
+    k.c = make_float4(xy.x, xy.y, zw.x, zw.y);
+    return k;
+}
 __device__ __forceinline__ float4 tf_classify(const TfView &tf, float v) {
-    const float u = fminf(fmaxf((v - tf.lo) * tf.du, 0.0f), 255.0f);
-    int i0;
-    floor_small(u, i0);
-    i0 = min(i0, 254);
-    const float fu = u - (float)i0;
-    const float4 c0 = __ldg(tf.rgba + i0), dc = __ldg(tf.drgba + i0);
-    return make_float4(fmaf(fu, dc.x, c0.x), fmaf(fu, dc.y, c0.y), fmaf(fu, dc.z, c0.z),
-                       fmaf(fu, dc.w, c0.w));
+    return classify(tf, v).c;
 }
 
 // Headlight Blinn-Phong coefficients (local lighting): rgb <- rgb (ka + kd n.L) +
@@ -367,8 +393,9 @@ struct Phong {
 
 // Value and gradient of the cubic B-spline at integer base ip with fractions f (derivative
 // weights d/df of the weights, the same taps).
-__device__ __forceinline__ float tricubic_grad_rep(const ReplView &rp, const int ip[3],
-                                                   const float f[3], float g[3]) {
+template <bool PACKED>
+__device__ __forceinline__ float tricubic_grad_of(const ReplView &rp, const int ip[3],
+                                                  const float f[3], float g[3]) {
     float wx[4], wy[4], wz[4], dx[4], dy[4], dz[4];
     bspline_w(f[0], wx);
     bspline_w(f[1], wy);
@@ -378,71 +405,53 @@ __device__ __forceinline__ float tricubic_grad_rep(const ReplView &rp, const int
     bspline_dw(f[2], dz);
     float s = 0.0f;
     g[0] = g[1] = g[2] = 0.0f;
-    if (rp.half) {  // two z at a time, as in tricubic_rep
-        const f32x2 sub = pack2(-rp.magic, -rp.magic);
-        f32x2 wx2[4], dx2[4];
+    const f32x2 sub = pack2(-rp.magic, -rp.magic);
+    f32x2 wx2[4], dx2[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            wx2[k] = pack2(wx[k], wx[k]);
-            dx2[k] = pack2(dx[k], dx[k]);
-        }
-        const uint4 *p = entry16(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
-        const unsigned row2 = 2u * rp.rnx, slice2 = row2 * rp.rny;
-#pragma unroll
-        for (int zh = 0; zh < 2; ++zh) {
-            f32x2 ps = 0ull, pdx = 0ull, pdy = 0ull;
-#pragma unroll
-            for (int yh = 0; yh < 2; ++yh) {
-                const uint4 *e = p + (zh ? slice2 : 0u) + (yh ? row2 : 0u);
-                const uint4 l = __ldg(e), u = __ldg(e + 1);
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const int b = 2 * yh + k;
-                    const f32x2 v0 = voxels2(k ? l.z : l.x, sub), v1 = voxels2(k ? l.w : l.y, sub);
-                    const f32x2 v2 = voxels2(k ? u.z : u.x, sub), v3 = voxels2(k ? u.w : u.y, sub);
-                    const f32x2 r =
-                        fma2(wx2[3], v3, fma2(wx2[2], v2, fma2(wx2[1], v1, mul2(wx2[0], v0))));
-                    const f32x2 rd =
-                        fma2(dx2[3], v3, fma2(dx2[2], v2, fma2(dx2[1], v1, mul2(dx2[0], v0))));
-                    const f32x2 wyb = pack2(wy[b], wy[b]);
-                    ps = fma2(wyb, r, ps);
-                    pdx = fma2(wyb, rd, pdx);
-                    pdy = fma2(pack2(dy[b], dy[b]), r, pdy);
-                }
-            }
-            const float2 p0 = unpack2(ps), p1 = unpack2(pdx), p2 = unpack2(pdy);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int c = 2 * zh + h;
-                s = fmaf(wz[c], h ? p0.y : p0.x, s);
-                g[0] = fmaf(wz[c], h ? p1.y : p1.x, g[0]);
-                g[1] = fmaf(wz[c], h ? p2.y : p2.x, g[1]);
-                g[2] = fmaf(dz[c], h ? p0.y : p0.x, g[2]);
-            }
-        }
-        return s;
+    for (int k = 0; k < 4; ++k) {
+        wx2[k] = pack2(wx[k], wx[k]);
+        dx2[k] = pack2(dx[k], dx[k]);
     }
-    float ps = 0.0f, pdx = 0.0f, pdy = 0.0f;
-    for_rows(rp, ip, [&](int c, int b, const float4 &v) {
-        float r = wx[0] * v.x;
-        r = fmaf(wx[1], v.y, r);
-        r = fmaf(wx[2], v.z, r);
-        r = fmaf(wx[3], v.w, r);
-        float rd = dx[0] * v.x;
-        rd = fmaf(dx[1], v.y, rd);
-        rd = fmaf(dx[2], v.z, rd);
-        rd = fmaf(dx[3], v.w, rd);
-        ps = fmaf(wy[b], r, ps);
-        pdx = fmaf(wy[b], rd, pdx);
-        pdy = fmaf(dy[b], r, pdy);
-        if (b < 3) return;
-        s = fmaf(wz[c], ps, s);
-        g[0] = fmaf(wz[c], pdx, g[0]);
-        g[1] = fmaf(wz[c], pdy, g[1]);
-        g[2] = fmaf(dz[c], ps, g[2]);
-        ps = pdx = pdy = 0.0f;
-    });
+    const char *p = first_entry<PACKED>(rp, ip);
+#pragma unroll
+    for (int zh = 0; zh < 2; ++zh) {
+        f32x2 ps = 0ull, pdx = 0ull, pdy = 0ull;
+#pragma unroll
+        for (int yh = 0; yh < 2; ++yh) {
+            Entry<PACKED> l, u;
+            l.load(entry_at<PACKED>(rp, p, 0, yh, zh));
+            u.load(entry_at<PACKED>(rp, p, 1, yh, zh));
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const int b = 2 * yh + k;
+                const f32x2 v0 = l.pair(2 * k, sub), v1 = l.pair(2 * k + 1, sub);
+                const f32x2 v2 = u.pair(2 * k, sub), v3 = u.pair(2 * k + 1, sub);
+                const f32x2 r =
+                    fma2(wx2[3], v3, fma2(wx2[2], v2, fma2(wx2[1], v1, mul2(wx2[0], v0))));
+                const f32x2 rd =
+                    fma2(dx2[3], v3, fma2(dx2[2], v2, fma2(dx2[1], v1, mul2(dx2[0], v0))));
+                const f32x2 wyb = pack2(wy[b], wy[b]);
+                ps = fma2(wyb, r, ps);
+                pdx = fma2(wyb, rd, pdx);
+                pdy = fma2(pack2(dy[b], dy[b]), r, pdy);
+            }
+        }
+        const float2 p0 = unpack2(ps), p1 = unpack2(pdx), p2 = unpack2(pdy);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = 2 * zh + h;
+            s = fmaf(wz[c], h ? p0.y : p0.x, s);
+            g[0] = fmaf(wz[c], h ? p1.y : p1.x, g[0]);
+            g[1] = fmaf(wz[c], h ? p2.y : p2.x, g[1]);
+            g[2] = fmaf(dz[c], h ? p0.y : p0.x, g[2]);
+        }
+    }
     return s;
+}
+__device__ __forceinline__ float tricubic_grad_rep(const ReplView &rp, const int ip[3],
+                                                   const float f[3], float g[3]) {
+    return rp.packed ? tricubic_grad_of<true>(rp, ip, f, g)
+                     : tricubic_grad_of<false>(rp, ip, f, g);
 }
 
 // Interpolation and classification variants (the paper's Fig. 4 comparison):

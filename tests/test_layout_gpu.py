@@ -1,5 +1,5 @@
-"""The render layouts of a resident volume at their edges: 16-bit volumes (packed 2^3 entries in
-two parity halves per row) and float32 ones (rows of 4), sizes from one voxel up, the whole range
+"""The render layouts of a resident volume at their edges: entries of 2^3 voxels in blocks of 2^3,
+16-bit ones packed, written in spans of a row: sizes from one voxel up, the whole range
 of each type, after an upload and after an update. Images within the suite's 1e-4 of the FP64
 oracle; the staged kernel reads another copy of the volume and must agree bit for bit."""
 import numpy as np
@@ -32,7 +32,7 @@ def R(torch):
 
 @pytest.mark.parametrize("dtype", [np.uint16, np.int16, np.float32])
 @pytest.mark.parametrize("shape", [(1, 1, 1), (1, 2, 3), (3, 1, 2), (2, 5, 4), (6, 7, 8),
-                                   (5, 4, 33), (3, 6, 132)])
+                                   (5, 4, 33), (3, 6, 132), (2, 3, 259), (3, 2, 523)])
 def test_layouts_of_every_size(R, orc, torch, shape, dtype):
     rng = np.random.default_rng(sum(shape))
     lo, hi = (0.0, 65535.0) if dtype == np.uint16 else (-32768.0, 32767.0)
