@@ -5,72 +5,39 @@
 //
 // It reads the checkpoints of a forward render (RenderLaunch::ckpt): the ray's last composited
 // sample and, for each segment of `seg` samples up to it, the transmittance at the segment's
-// start (-1 for segments without a composited sample). Given those, the segments of a ray are
-// independent but for what lies behind each, so a group of G lanes takes one ray and its
-// lanes take G consecutive segments at a time, back to front:
-//   1. each lane recomputes its segment forward from the checkpoint (never dividing by
-//      1 - alpha), keeping every sample's value and transmittance, and also composites the
-//      segment on its own from transmittance 1, P = (C, T);
-//   2. a scan of the "over" operator across the group gives each lane what lies behind its
-//      segment -- the segments of the lanes after it in this round, then the carry of the
-//      rounds before -- as S = normalised colour behind, U = transmittance behind;
-//   3. each lane walks its samples back to front:
+// start (-1 for segments without composited samples). One warp takes one ray and walks its
+// segments back to front, a block of 32 consecutive samples at a time, a lane per sample:
+//   1. forward over the segment's blocks: every lane resamples and classifies its sample, and a
+//      prefix product from the checkpoint gives its transmittance T_j (never dividing by
+//      1 - alpha);
+//   2. back over the blocks: a suffix scan of the "over" operator gives each lane what lies
+//      behind its sample -- the rest of the block, then the carry of the blocks before -- as
+//      S = normalised colour behind, U = transmittance behind, and
 //        dL/drgb_j   = T_j alpha_j g_rgb
 //        dL/dalpha_j = T_j [ g_rgb . (rgb_j - S) + g_A U ]
-//        S <- alpha_j rgb_j + (1 - alpha_j) S,   U <- (1 - alpha_j) U
-//      and chains through alpha = 1 - (1-a)^delta, the table interpolation (into the two
-//      entries) and the 64 B-spline taps (into the voxels).
-// A long ray then costs about 1/G of its segments in serial steps. Transfer-function
-// gradients are summed in shared memory per CTA, voxel gradients with global float atomics
-// (the summation order, and so the last bits, vary from run to run). Samples in empty bricks
-// or clear cells (opacity exactly zero, whose derivative is taken as zero at the clamp, so
-// that every contribution of such a sample is exactly zero) are skipped exactly as in the
+//      chained through alpha = 1 - (1-a)^delta, the table interpolation (into the two entries)
+//      and the 64 B-spline taps (into the voxels);
+//   3. the lanes' contributions are summed in shared memory, sample by sample, the warp's lanes
+//      being the taps (two each) and the table components: no two lanes meet at an address, so
+//      plain adds do. Voxels collect in a box of up to ADJ_BOX floats around 16 consecutive
+//      samples, which then goes to the volume as float4 atomics.
+// Transfer-function gradients are kept per warp and added up per CTA (global float atomics at
+// the end: the summation order, and so the last bits, vary from run to run). Samples in empty
+// bricks or clear cells (opacity exactly zero, whose derivative is taken as zero at the clamp,
+// so that every contribution of such a sample is exactly zero) are skipped exactly as in the
 // forward.
+//
+// What bounds it: adding every tap to the volume on its own was bound by the vector atomics of
+// L2 (16 rows a sample of one float4, two float2 or float + float2 + float, 2.25 atomics a row
+// on average, at 192 G/s measured: 36 a sample), and eight shared-memory atomics a sample
+// contended for the few table entries in use. Consecutive samples half a voxel apart share most
+// of their taps, so a box of 16 gives some 4.9 atomic sectors a sample instead. 256^3 float32 at
+// 512^2, soft tissue visible (17 M samples): 1.92 ms a view against 4.0 ms. What bounds it now is
+// the chain of a warp's adds and the registers (16 warps an SM): 54% of the issue slots, 61% of
+// the L1 and shared-memory data path.
 #include "vrc_internal.h"
 
 namespace vrc {
-
-constexpr int ADJ_WARPS = 4;
-// Lanes per ray: more lanes shorten a ray's serial chain of segments, fewer keep more rays in
-// flight. Measured per launch (ms; 256^3 float32 CT without termination / 512^2 x 2000 int16
-// CT at step 0.25 with termination):
-//   image        1 lane   2      4      8
-//   256^2        1.14     0.82   0.61   0.34
-//   512^2        1.36     1.07   0.70   0.63
-//   1024^2       2.02     1.53   1.42   1.81    (512^2 x 2000: 2.08 1.78 1.55 1.62)
-//   2048^2       3.92     3.70   4.58   6.76
-//   4096^2 (512^2 x 2000)  7.92   7.53   9.99  15.2
-__host__ __device__ constexpr int adjoint_lanes_for(long pixels) {
-    return pixels < (512L << 10) ? 8 : pixels < (2048L << 10) ? 4 : 2;
-}
-
-struct SampleEval {
-    float s;        // resampled value
-    float u_raw;    // index coordinate before clamping
-    int i0;         // lower table entry
-    float fu;       // weight of the upper entry
-    float4 rgba;    // interpolated table value (alpha before clamping)
-    float4 drgba;   // table difference at i0
-    float alpha;    // segment opacity
-};
-
-__device__ __forceinline__ void eval_sample(const RenderLaunch &L, const int ip[3],
-                                            const float f[3], float delta, SampleEval &e) {
-    e.s = tricubic_rep(L.rep, ip, f);
-    e.u_raw = (e.s - L.tf.lo) * L.tf.du;
-    const float u = fminf(fmaxf(e.u_raw, 0.0f), 255.0f);
-    int i0;
-    floor_small(u, i0);
-    e.i0 = min(i0, 254);
-    e.fu = u - (float)e.i0;
-    const float4 c0 = __ldg(L.tf.tab + 2 * e.i0);
-    e.drgba = __ldg(L.tf.tab + 2 * e.i0 + 1);
-    e.rgba.x = fmaf(e.fu, e.drgba.x, c0.x);
-    e.rgba.y = fmaf(e.fu, e.drgba.y, c0.y);
-    e.rgba.z = fmaf(e.fu, e.drgba.z, c0.z);
-    e.rgba.w = fmaf(e.fu, e.drgba.w, c0.w);
-    e.alpha = segment_alpha(e.rgba.w, delta);
-}
 
 // Adds (v0, v1, v2, v3) to the voxel gradients of taps x0 .. x0+3 of a row, clamped to
 // [0, nx-1], with the fewest aligned vector atomics (one float4, two float2 or float + float2
@@ -100,218 +67,336 @@ __device__ __forceinline__ void add_taps_x(float *row, int x0, int nx, float v0,
     atomicAdd(row + min(max(x0 + 3, 0), nx - 1), v3);
 }
 
-template <bool ESL, bool VOLGRAD, int ADJ_G>
-__global__ void __launch_bounds__(32 * ADJ_WARPS) adjoint_kernel(AdjointLaunch A) {
-    __shared__ float s_gtf[256 * 4];
-    for (int i = threadIdx.x; i < 1024; i += blockDim.x) s_gtf[i] = 0.0f;
-    __syncthreads();
-    const RenderLaunch &L = A.L;
+constexpr int ADJ_WARPS = 4;
+constexpr int ADJ_BOX = 1152;    // floats of a warp's box of voxel gradients
+constexpr int ADJ_CHUNK = 16;    // samples summed into one box
+constexpr int ADJ_REC = 36;      // words of a sample's record (conflict-free 16-byte stores)
+constexpr int ADJ_TILE = 32;     // pixels of a CTA at most
 
-    // ADJ_G lanes per ray: a warp takes a row of 32 / ADJ_G pixels, a CTA ADJ_WARPS such rows
-    // (ADJ_G from adjoint_lanes_for: the image's pixel count)
-    constexpr int G = ADJ_G, RX = 32 / ADJ_G;
+// A ray of the CTA's tile that composited something.
+struct AdjRay {
+    RayPos rp;
+    float4 g;        // dL/d(pixel)
+    int pix, k0, jlast;
+};
+
+struct alignas(16) AdjWarp {  // a warp's shared memory
+    float box[ADJ_BOX];
+    float tf[1024];
+    // per sample of the chunk: 16 products wx[a] wy[b]; (ds wz[0], ds wz[2], box offset of the
+    // first tap, table offset); the same with wz[1], wz[3]; the 8 table components
+    float rec[(ADJ_CHUNK + 1) * ADJ_REC];
+};
+
+// NB: blocks of 32 samples that a segment spans at most.
+template <bool ESL, bool VOLGRAD, int NB>
+__global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunch A, int tw_shift,
+                                                                    int th_shift) {
+    __shared__ AdjWarp s_warp[ADJ_WARPS];
+    __shared__ AdjRay s_ray[ADJ_TILE];
+    __shared__ int s_count, s_head;
+    const RenderLaunch &L = A.L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int q = lane & (G - 1), gbase = lane & ~(G - 1);
-    const unsigned gmask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << gbase);
-    const int tiles_x = (L.cam.width + RX - 1) / RX;
-    const int px = (blockIdx.x % tiles_x) * RX + lane / G;
-    const int py = (blockIdx.x / tiles_x) * ADJ_WARPS + warp;
     const float step = L.grid.step;
     const int seg = A.seg;
+    if (threadIdx.x == 0) s_count = s_head = 0;
+    __syncthreads();
 
-    // the forward's record of this ray: first checkpointed segment, last composited sample
-    // (read first: most rays of a CT view composite nothing and need no set-up)
-    bool work = false;
-    float4 g = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    int2 h = make_int2(0, -1);
-    if (px < L.cam.width && py < L.cam.height) {
-        g = A.grad_out[(long)py * L.cam.width + px];
-        if (g.x != 0.0f || g.y != 0.0f || g.z != 0.0f || g.w != 0.0f) {
-            h = L.ckpt_head[(long)py * L.cam.width + px];
-            work = h.y >= 0;
-        }
-    }
-    RaySetup ray;
-    ray.nseg = 0;
-    if (work) ray_setup(L.cam, L.grid, px, py, ray);
-    RayPos rp;
-    ray_pos_init(ray, step, rp);
-    float Pf[3], df[3], inv_df[3];
-    ray_float(rp, Pf, df, inv_df);
-    const uint8_t *dist = nullptr;
-    if (ESL)
-        dist = L.dist + (long)octant_of(df) * L.bricks.nb[0] * L.bricks.nb[1] * L.bricks.nb[2];
-    const int k0 = work ? max(h.x, 0) : 0;
-    const int jlast = work ? min(h.y, rp.nseg - 1) : -1;
-    const float *ck_row = L.ckpt + ((long)py * L.cam.width + px) * L.ckpt_K;
-    const int klast = jlast >= 0 ? min(jlast / seg, L.ckpt_K - 1) : -1;
-
-    float buf_s[ADJ_MAX_SEG], buf_T[ADJ_MAX_SEG];
-    int buf_j[ADJ_MAX_SEG];
-    // what lies behind the segments of the current round: normalised colour and transmittance
-    float cS0 = 0.0f, cS1 = 0.0f, cS2 = 0.0f, cU = 1.0f;
-    // rounds of G segments, back to front: lane q takes segment kr - q
-    for (int kr = klast; kr >= k0; kr -= G) {
-        const int k = kr - q;
-        float T = k >= k0 ? ck_row[k] : -1.0f;
-        // recompute the segment forward from its checkpoint (absolute transmittance T) and
-        // from 1 (its own composite over what lies behind it)
-        int n = 0;
-        float l0 = 0.0f, l1 = 0.0f, l2 = 0.0f, lT = 1.0f;
-        if (T >= 0.0f) {  // else no composited sample in this segment
-            const int j1 = min(k * seg + seg, jlast + 1);
-            for (int j = k * seg; j < j1; ++j) {
-                int ip[3];
-                float f[3], delta;
-                place(rp, step, L.grid.n, j, ip, f, delta);
-                if (ESL && (dist[brick_of(L.bricks, ip)] != 0 ||
-                            (L.cells && !cell_open(L.cells, L.grid.n, ip))))
-                    continue;
-                SampleEval e;
-                eval_sample(L, ip, f, delta, e);
-                buf_s[n] = e.s;
-                buf_T[n] = T;
-                buf_j[n] = j;
-                ++n;
-                T = T - T * e.alpha;
-                const float w = lT * e.alpha;
-                l0 = fmaf(w, e.rgba.x, l0);
-                l1 = fmaf(w, e.rgba.y, l1);
-                l2 = fmaf(w, e.rgba.z, l2);
-                lT = lT - w;
-            }
-        }
-        // behind lane q's segment: the segments of lanes q-1 .. 0 of this round (front to
-        // back), then the carry. Inclusive scan v_q = P_q o P_{q-1} o ... o P_0 of the "over"
-        // operator (C_a, T_a) o (C_b, T_b) = (C_a + T_a C_b, T_a T_b).
-        float v0 = l0, v1 = l1, v2 = l2, vT = lT;
-        for (int o = 1; o < G; o <<= 1) {
-            const float p0 = __shfl_up_sync(gmask, v0, o, G);
-            const float p1 = __shfl_up_sync(gmask, v1, o, G);
-            const float p2 = __shfl_up_sync(gmask, v2, o, G);
-            const float pT = __shfl_up_sync(gmask, vT, o, G);
-            if (q >= o) {
-                v0 = fmaf(vT, p0, v0);
-                v1 = fmaf(vT, p1, v1);
-                v2 = fmaf(vT, p2, v2);
-                vT = vT * pT;
-            }
-        }
-        float e0 = __shfl_up_sync(gmask, v0, 1, G), e1 = __shfl_up_sync(gmask, v1, 1, G);
-        float e2 = __shfl_up_sync(gmask, v2, 1, G), eT = __shfl_up_sync(gmask, vT, 1, G);
-        if (q == 0) {
-            e0 = e1 = e2 = 0.0f;
-            eT = 1.0f;
-        }
-        float S0 = fmaf(eT, cS0, e0), S1 = fmaf(eT, cS1, e1), S2 = fmaf(eT, cS2, e2);
-        float U = eT * cU;
-        {  // the next round lies in front of this one: carry = v_{G-1} o carry
-            const float a0 = __shfl_sync(gmask, v0, G - 1, G);
-            const float a1 = __shfl_sync(gmask, v1, G - 1, G);
-            const float a2 = __shfl_sync(gmask, v2, G - 1, G);
-            const float aT = __shfl_sync(gmask, vT, G - 1, G);
-            cS0 = fmaf(aT, cS0, a0);
-            cS1 = fmaf(aT, cS1, a1);
-            cS2 = fmaf(aT, cS2, a2);
-            cU = aT * cU;
-        }
-        // back to front over the segment
-        for (int i = n - 1; i >= 0; --i) {
-            int ip[3];
-            float f[3], delta;
-            place(rp, step, L.grid.n, buf_j[i], ip, f, delta);
-            // classification from the stored value (as in eval_sample)
-            const float s = buf_s[i];
-            const float u_raw = (s - L.tf.lo) * L.tf.du;
-            const float u = fminf(fmaxf(u_raw, 0.0f), 255.0f);
-            int i0;
-            floor_small(u, i0);
-            i0 = min(i0, 254);
-            const float fu = u - (float)i0;
-            const float4 c0 = __ldg(L.tf.tab + 2 * i0), dc = __ldg(L.tf.tab + 2 * i0 + 1);
-            const float r = fmaf(fu, dc.x, c0.x), gg = fmaf(fu, dc.y, c0.y);
-            const float b = fmaf(fu, dc.z, c0.z), araw = fmaf(fu, dc.w, c0.w);
-            const float a = fminf(fmaxf(araw, 0.0f), ALPHA_MAX);
-            const float alpha = segment_alpha(araw, delta);
-            const float Tj = buf_T[i];
-            // compositing
-            const float ta = Tj * alpha;
-            const float d_r = ta * g.x, d_g = ta * g.y, d_b = ta * g.z;
-            const float dalpha =
-                Tj * (g.x * (r - S0) + g.y * (gg - S1) + g.z * (b - S2) + g.w * U);
-            // opacity correction (zero derivative at the clamp ends; from above at 0 when
-            // asked)
-            const bool up = araw > 0.0f || (A.open_alpha && araw == 0.0f);
-            const float da = (up && araw <= ALPHA_MAX)
-                                 ? delta * exp2f((delta - 1.0f) * __log2f(1.0f - a))
-                                 : 0.0f;
-            const float d_a = dalpha * da;
-            // table interpolation
-            const float w1 = fu, w0 = 1.0f - fu;
-            float *t0 = s_gtf + 4 * i0;
-            atomicAdd(t0 + 0, w0 * d_r);
-            atomicAdd(t0 + 1, w0 * d_g);
-            atomicAdd(t0 + 2, w0 * d_b);
-            atomicAdd(t0 + 3, w0 * d_a);
-            atomicAdd(t0 + 4, w1 * d_r);
-            atomicAdd(t0 + 5, w1 * d_g);
-            atomicAdd(t0 + 6, w1 * d_b);
-            atomicAdd(t0 + 7, w1 * d_a);
-            // resampling taps
-            if (VOLGRAD && u_raw > 0.0f && u_raw < 255.0f) {
-                const float ds = (d_r * dc.x + d_g * dc.y + d_b * dc.z + d_a * dc.w) * L.tf.du;
-                if (ds != 0.0f) {
-                    float wx[4], wy[4], wz[4];
-                    bspline_w(f[0], wx);
-                    bspline_w(f[1], wy);
-                    bspline_w(f[2], wz);
-                    const int nx = L.grid.n[0], ny = L.grid.n[1], nz = L.grid.n[2];
-#pragma unroll
-                    for (int cz = 0; cz < 4; ++cz) {
-                        const int z = min(max(ip[2] - 1 + cz, 0), nz - 1);
-                        const float wzc = wz[cz] * ds;
-#pragma unroll
-                        for (int cy = 0; cy < 4; ++cy) {
-                            const int y = min(max(ip[1] - 1 + cy, 0), ny - 1);
-                            const float wyz = wy[cy] * wzc;
-                            float *row = A.grad_vol + ((long)z * ny + y) * nx;
-                            add_taps_x(row, ip[0] - 1, nx, wx[0] * wyz, wx[1] * wyz,
-                                       wx[2] * wyz, wx[3] * wyz);
-                        }
-                    }
+    // the tile's rays that have work, by the forward's record: first checkpointed segment, last
+    // composited sample (read first: most rays of a CT view composite nothing and need no set-up)
+    if (threadIdx.x < (1u << (tw_shift + th_shift))) {
+        const int tiles_x = (L.cam.width + (1 << tw_shift) - 1) >> tw_shift;
+        const int px = ((blockIdx.x % tiles_x) << tw_shift) + (threadIdx.x & ((1 << tw_shift) - 1));
+        const int py = ((blockIdx.x / tiles_x) << th_shift) + (threadIdx.x >> tw_shift);
+        if (px < L.cam.width && py < L.cam.height) {
+            const int pix = py * L.cam.width + px;
+            const float4 g = A.grad_out[pix];
+            const int2 h = L.ckpt_head[pix];
+            if (h.y >= 0 && (g.x != 0.0f || g.y != 0.0f || g.z != 0.0f || g.w != 0.0f)) {
+                RaySetup ray;
+                ray_setup(L.cam, L.grid, px, py, ray);
+                if (ray.nseg > 0) {
+                    AdjRay r;
+                    ray_pos_init(ray, step, r.rp);
+                    r.g = g;
+                    r.pix = pix;
+                    r.k0 = max(h.x, 0);
+                    r.jlast = min(h.y, r.rp.nseg - 1);
+                    s_ray[atomicAdd(&s_count, 1)] = r;
                 }
             }
-            S0 = fmaf(alpha, r - S0, S0);
-            S1 = fmaf(alpha, gg - S1, S1);
-            S2 = fmaf(alpha, b - S2, S2);
-            U = U - alpha * U;
+        }
+    }
+    __syncthreads();
+    const int count = s_count;
+    if (count == 0) return;
+
+    AdjWarp &W = s_warp[warp];
+    for (int i = lane; i < ADJ_BOX; i += 32) W.box[i] = 0.0f;
+    for (int i = lane; i < 1024; i += 32) W.tf[i] = 0.0f;
+    __syncwarp();
+    const int nx = L.grid.n[0], ny = L.grid.n[1], nz = L.grid.n[2];
+    // rows of the volume's gradient on 16-byte boundaries
+    const bool aligned = VOLGRAD && (nx & 3) == 0 && ((uintptr_t)A.grad_vol & 15) == 0;
+    const long nbricks = ESL ? (long)L.bricks.nb[0] * L.bricks.nb[1] * L.bricks.nb[2] : 0;
+
+    while (true) {
+        int qi = 0;
+        if (lane == 0) qi = atomicAdd(&s_head, 1);
+        qi = __shfl_sync(0xffffffffu, qi, 0);
+        if (qi >= count) break;
+        const RayPos rp = s_ray[qi].rp;
+        const float4 g = s_ray[qi].g;
+        const int k0 = s_ray[qi].k0, jlast = s_ray[qi].jlast;
+        const float df[3] = {rp.d[0].hi, rp.d[1].hi, rp.d[2].hi};
+        const uint8_t *dist = ESL ? L.dist + octant_of(df) * nbricks : nullptr;
+        const float *ck_row = L.ckpt + (long)s_ray[qi].pix * L.ckpt_K;
+        // what lies behind the current block: normalised colour and transmittance
+        float cS0 = 0.0f, cS1 = 0.0f, cS2 = 0.0f, cU = 1.0f;
+        for (int k = min(jlast / seg, L.ckpt_K - 1); k >= k0; --k) {
+            const float Tk = ck_row[k];
+            if (!(Tk >= 0.0f)) continue;  // no composited sample in this segment
+            const int j1 = min(k * seg + seg, jlast + 1);
+            int chunk = ADJ_CHUNK;
+            // forward: values, opacities and transmittances of the segment's samples
+            int ip[NB][3];
+            float f[NB][3], sv[NB], Tj[NB];
+            unsigned live_bits[NB];
+            float T = Tk;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const int j = k * seg + 32 * b + lane;
+                bool live = j < j1;
+                float delta, eT = 1.0f;
+                sv[b] = 0.0f;
+                if (live) {
+                    place(rp, step, L.grid.n, j, ip[b], f[b], delta);
+                    if (ESL && (dist[brick_of(L.bricks, ip[b])] != 0 ||
+                                (L.cells && !cell_open(L.cells, L.grid.n, ip[b]))))
+                        live = false;
+                }
+                if (live) {
+                    sv[b] = tricubic_rep(L.rep, ip[b], f[b]);
+                    eT = 1.0f - segment_alpha(classify(L.tf, sv[b]).c.w, delta);
+                }
+                live_bits[b] = __ballot_sync(0xffffffffu, live);
+                if (live_bits[b] == 0u) continue;
+                float incl = eT;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float p = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl = p * incl;
+                }
+                const float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+                Tj[b] = lane == 0 ? T : T * excl;
+                T = T * __shfl_sync(0xffffffffu, incl, 31);
+            }
+            // back to front over the blocks
+#pragma unroll
+            for (int b = NB - 1; b >= 0; --b) {
+                if (live_bits[b] == 0u) continue;
+                const bool live = (live_bits[b] >> lane) & 1u;
+                const int j = k * seg + 32 * b + lane;
+                const float delta = j < rp.nseg - 1 ? step : rp.dlast;
+                const Classified c = classify(L.tf, sv[b]);
+                const float alpha = live ? segment_alpha(c.c.w, delta) : 0.0f;
+                // behind the sample: suffix scan of v_j = P_j o ... o P_31 of the "over" operator
+                // (C_a, T_a) o (C_b, T_b) = (C_a + T_a C_b, T_a T_b)
+                float v0 = alpha * c.c.x, v1 = alpha * c.c.y, v2 = alpha * c.c.z, vT = 1.0f - alpha;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const float p0 = __shfl_down_sync(0xffffffffu, v0, o);
+                    const float p1 = __shfl_down_sync(0xffffffffu, v1, o);
+                    const float p2 = __shfl_down_sync(0xffffffffu, v2, o);
+                    const float pT = __shfl_down_sync(0xffffffffu, vT, o);
+                    if (lane + o < 32) {
+                        v0 = fmaf(vT, p0, v0);
+                        v1 = fmaf(vT, p1, v1);
+                        v2 = fmaf(vT, p2, v2);
+                        vT = vT * pT;
+                    }
+                }
+                float S0 = __shfl_down_sync(0xffffffffu, v0, 1);
+                float S1 = __shfl_down_sync(0xffffffffu, v1, 1);
+                float S2 = __shfl_down_sync(0xffffffffu, v2, 1);
+                float U = __shfl_down_sync(0xffffffffu, vT, 1);
+                if (lane == 31) {
+                    S0 = S1 = S2 = 0.0f;
+                    U = 1.0f;
+                }
+                S0 = fmaf(U, cS0, S0);
+                S1 = fmaf(U, cS1, S1);
+                S2 = fmaf(U, cS2, S2);
+                U = U * cU;
+                {  // the next block lies in front of this one: carry = v_0 o carry
+                    const float aT = __shfl_sync(0xffffffffu, vT, 0);
+                    cS0 = fmaf(aT, cS0, __shfl_sync(0xffffffffu, v0, 0));
+                    cS1 = fmaf(aT, cS1, __shfl_sync(0xffffffffu, v1, 0));
+                    cS2 = fmaf(aT, cS2, __shfl_sync(0xffffffffu, v2, 0));
+                    cU = aT * cU;
+                }
+                // compositing
+                const float ta = Tj[b] * alpha;
+                const float d_r = ta * g.x, d_g = ta * g.y, d_b = ta * g.z;
+                const float dalpha = Tj[b] * (g.x * (c.c.x - S0) + g.y * (c.c.y - S1) +
+                                              g.z * (c.c.z - S2) + g.w * U);
+                // opacity correction (zero derivative at the clamp ends; from above at 0 when
+                // asked)
+                const float a = fminf(fmaxf(c.c.w, 0.0f), ALPHA_MAX);
+                const bool up = c.c.w > 0.0f || (A.open_alpha && c.c.w == 0.0f);
+                const float da = (up && c.c.w <= ALPHA_MAX)
+                                     ? delta * exp2f((delta - 1.0f) * __log2f(1.0f - a))
+                                     : 0.0f;
+                const float d_a = dalpha * da;
+                float ds = 0.0f;
+                if (VOLGRAD && live && c.u_raw > 0.0f && c.u_raw < 255.0f)
+                    ds = (d_r * c.dc.x + d_g * c.dc.y + d_b * c.dc.z + d_a * c.dc.w) * L.tf.du;
+                const unsigned vox = VOLGRAD ? __ballot_sync(0xffffffffu, ds != 0.0f) : 0u;
+
+                for (int l0 = 0; l0 < 32;) {
+                    const unsigned span = (chunk == 32 ? 0xffffffffu : (1u << chunk) - 1u) << l0;
+                    unsigned todo = live_bits[b] & span;
+                    if (todo == 0u) {
+                        l0 += chunk;
+                        continue;
+                    }
+                    const bool mine = (todo >> lane) & 1u;
+                    // box of the taps, from x0 (a multiple of 4), y0, z0
+                    int x0 = 0, y0 = 0, z0 = 0, px = 0, ey = 0, ez = 0, plane = 0;
+                    if (VOLGRAD && (vox & span)) {
+                        const bool v = mine && ds != 0.0f;
+                        const int big = 1 << 20;
+                        x0 = (__reduce_min_sync(0xffffffffu, v ? ip[b][0] : big) - 1) & ~3;
+                        y0 = __reduce_min_sync(0xffffffffu, v ? ip[b][1] : big) - 1;
+                        z0 = __reduce_min_sync(0xffffffffu, v ? ip[b][2] : big) - 1;
+                        px = (__reduce_max_sync(0xffffffffu, v ? ip[b][0] : -big) + 6 - x0) & ~3;
+                        ey = __reduce_max_sync(0xffffffffu, v ? ip[b][1] : -big) + 3 - y0;
+                        ez = __reduce_max_sync(0xffffffffu, v ? ip[b][2] : -big) + 3 - z0;
+                        // rows and planes 4-float groups apart from each other in the banks
+                        if (px == 16) px = 20;
+                        plane = px * ey;
+                        plane += ((px == 8 ? 4 : 16) - plane) & 31;
+                        if (plane * ez > ADJ_BOX) {  // long steps: fewer samples a box (one
+                            chunk >>= 1;             // sample takes 8 x 4 x 4 at most)
+                            continue;
+                        }
+                    }
+                    const bool boxed = plane != 0;
+                    if (mine) {  // the chunk's records, without gaps
+                        float *r = W.rec + __popc(todo & ((1u << lane) - 1u)) * ADJ_REC;
+                        if (VOLGRAD && boxed) {
+                            float wx[4], wy[4], wz[4];
+                            bspline_w(f[b][0], wx);
+                            bspline_w(f[b][1], wy);
+                            bspline_w(f[b][2], wz);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                *(float4 *)(r + 4 * i) = make_float4(wx[0] * wy[i], wx[1] * wy[i],
+                                                                     wx[2] * wy[i], wx[3] * wy[i]);
+                            // a sample without a voxel gradient adds zeros at the box's start
+                            const float o = __int_as_float(
+                                ds == 0.0f ? 0 : (ip[b][2] - 1 - z0) * plane +
+                                                     (ip[b][1] - 1 - y0) * px + (ip[b][0] - 1 - x0));
+                            *(float4 *)(r + 16) = make_float4(wz[0] * ds, wz[2] * ds, o, 0.0f);
+                            *(float4 *)(r + 20) = make_float4(wz[1] * ds, wz[3] * ds, o, 0.0f);
+                        }
+                        r[19] = __int_as_float(4 * c.i0);
+                        const float w1 = c.fu, w0 = 1.0f - c.fu;
+                        *(float4 *)(r + 24) = make_float4(w0 * d_r, w0 * d_g, w0 * d_b, w0 * d_a);
+                        *(float4 *)(r + 28) = make_float4(w1 * d_r, w1 * d_g, w1 * d_b, w1 * d_a);
+                    }
+                    __syncwarp();
+                    // sample by sample: lane (a, b, h) adds the taps (a, b, h) and (a, b, h + 2),
+                    // lanes 0 .. 7 the table components; the next record is read ahead
+                    const int n = __popc(todo);
+                    const float *r = W.rec;
+                    if (VOLGRAD && boxed) {
+                        float *t0 = W.box + (lane & 3) + ((lane >> 2) & 3) * px +
+                                    (lane >> 4) * plane;
+                        const float *rw = r + (lane & 15), *rz = r + 16 + 4 * (lane >> 4);
+                        const float *re = r + 24 + (lane & 7);
+                        float w = *rw, e = *re;
+                        float4 z = *(const float4 *)rz;
+#pragma unroll 2
+                        for (int i = 1; i <= n; ++i) {
+                            // (the record after the last is read too, and not used)
+                            const float w2 = rw[i * ADJ_REC], e2 = re[i * ADJ_REC];
+                            const float4 z2 = *(const float4 *)(rz + i * ADJ_REC);
+                            float *t = t0 + __float_as_int(z.z);
+                            const float u0 = t[0], u1 = t[2 * plane];
+                            t[0] = fmaf(w, z.x, u0);
+                            t[2 * plane] = fmaf(w, z.y, u1);
+                            if (lane < 8) W.tf[__float_as_int(z.w) + lane] += e;
+                            __syncwarp();
+                            w = w2;
+                            e = e2;
+                            z = z2;
+                        }
+                    } else {
+                        for (int i = 0; i < n; ++i) {
+                            if (lane < 8)
+                                W.tf[__float_as_int(r[i * ADJ_REC + 19]) + lane] +=
+                                    r[i * ADJ_REC + 24 + lane];
+                            __syncwarp();
+                        }
+                    }
+                    if (VOLGRAD && boxed) {
+                        // the box to the volume, 4 voxels along x a lane and a few rows a step,
+                        // and back to zeros
+                        const int pq = px >> 2, per = 32 / pq, q = lane % pq;
+                        int yy = lane / pq, zz = 0;
+                        if (yy >= per) yy = 1 << 20;
+                        for (int row = yy; row < ey * ez; row += per, yy += per) {
+                            while (yy >= ey) {
+                                yy -= ey;
+                                ++zz;
+                            }
+                            float4 *cell = (float4 *)(W.box + zz * plane + yy * px + 4 * q);
+                            const float4 v = *cell;
+                            if (v.x == 0.0f && v.y == 0.0f && v.z == 0.0f && v.w == 0.0f) continue;
+                            *cell = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                            const int y = min(max(y0 + yy, 0), ny - 1);
+                            const int z = min(max(z0 + zz, 0), nz - 1);
+                            const int x = x0 + 4 * q;
+                            float *to = A.grad_vol + ((long)z * ny + y) * nx;
+                            if (aligned && x >= 0 && x + 3 < nx) atomicAdd((float4 *)(to + x), v);
+                            else add_taps_x(to, x, nx, v.x, v.y, v.z, v.w);
+                        }
+                        __syncwarp();
+                    }
+                    l0 += chunk;
+                }
+            }
         }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < 1024; i += blockDim.x) {
-        const float v = s_gtf[i];
+        float v = 0.0f;
+#pragma unroll
+        for (int w = 0; w < ADJ_WARPS; ++w) v += s_warp[w].tf[i];
         if (v != 0.0f) atomicAdd(A.grad_tf + i, v);
     }
 }
 
-template <int G>
-static void launch_adjoint_g(const AdjointLaunch &A, cudaStream_t st) {
-    constexpr int RX = 32 / G;
-    const unsigned grid = (unsigned)(((long)(A.L.cam.width + RX - 1) / RX) *
-                                     ((A.L.cam.height + ADJ_WARPS - 1) / ADJ_WARPS));
+template <int NB>
+static void launch_adjoint_n(const AdjointLaunch &A, cudaStream_t st) {
+    // a tile of 8 x 4 pixels a CTA, or 4 x 2 where 8 x 4 would leave SMs without one
+    const long pixels = (long)A.L.cam.width * A.L.cam.height;
+    const int tw = pixels < 64 * 1024 ? 2 : 3, th = tw - 1;
+    const unsigned grid = (unsigned)((((long)A.L.cam.width + (1 << tw) - 1) >> tw) *
+                                     ((A.L.cam.height + (1 << th) - 1) >> th));
     const bool esl = A.L.dist != nullptr, vg = A.grad_vol != nullptr;
-    if (esl && vg) adjoint_kernel<true, true, G><<<grid, 32 * ADJ_WARPS, 0, st>>>(A);
-    else if (esl) adjoint_kernel<true, false, G><<<grid, 32 * ADJ_WARPS, 0, st>>>(A);
-    else if (vg) adjoint_kernel<false, true, G><<<grid, 32 * ADJ_WARPS, 0, st>>>(A);
-    else adjoint_kernel<false, false, G><<<grid, 32 * ADJ_WARPS, 0, st>>>(A);
+    if (esl && vg) adjoint_kernel<true, true, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
+    else if (esl) adjoint_kernel<true, false, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
+    else if (vg) adjoint_kernel<false, true, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
+    else adjoint_kernel<false, false, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
 }
 
 cudaError_t launch_adjoint(const AdjointLaunch &A, cudaStream_t st) {
-    switch (adjoint_lanes_for((long)A.L.cam.width * A.L.cam.height)) {
-    case 8: launch_adjoint_g<8>(A, st); break;
-    case 4: launch_adjoint_g<4>(A, st); break;
-    default: launch_adjoint_g<2>(A, st);
-    }
+    static_assert(ADJ_MAX_SEG <= 128, "a segment spans at most 4 blocks of 32 samples");
+    if (A.seg <= 32) launch_adjoint_n<1>(A, st);
+    else if (A.seg <= 64) launch_adjoint_n<2>(A, st);
+    else launch_adjoint_n<4>(A, st);
     return cudaGetLastError();
 }
 
