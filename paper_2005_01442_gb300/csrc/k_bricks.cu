@@ -555,6 +555,34 @@ cudaError_t launch_cellmask(const VolView &v, int B, const int nb[3], const uint
     return cudaGetLastError();
 }
 
+// One thread per tile: the cells 8t .. 8t + 7 are the blocks 2t + 1 and 2t + 2 (cell_open), those
+// of tile 0 and the cell -1 the blocks 0 .. 2.
+__global__ void __launch_bounds__(256) tile_occupancy_kernel(const uint2 *__restrict__ cells,
+                                                             int nfx, int nfy, int nfz, int ntx,
+                                                             int nty, int ntz,
+                                                             uint8_t *__restrict__ tiles) {
+    const long i = (long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= (long)ntx * nty * ntz) return;
+    const int tx = (int)(i % ntx), ty = (int)((i / ntx) % nty), tz = (int)(i / ((long)ntx * nty));
+    uint32_t any = 0u;
+    for (int z = tz ? 2 * tz + 1 : 0; z < min(2 * tz + 3, nfz); ++z)
+        for (int y = ty ? 2 * ty + 1 : 0; y < min(2 * ty + 3, nfy); ++y)
+            for (int x = tx ? 2 * tx + 1 : 0; x < min(2 * tx + 3, nfx); ++x) {
+                const uint2 w = __ldg(cells + ((long)z * nfy + y) * nfx + x);
+                any |= w.x | w.y;
+            }
+    tiles[i] = any ? 1 : 0;
+}
+
+cudaError_t launch_tile_occupancy(const uint32_t *cells, const int n[3], const int nt[3],
+                                  uint8_t *tiles, cudaStream_t st) {
+    const long count = (long)nt[0] * nt[1] * nt[2];
+    tile_occupancy_kernel<<<(unsigned)((count + 255) / 256), 256, 0, st>>>(
+        (const uint2 *)cells, cell_blocks(n[0]), cell_blocks(n[1]), cell_blocks(n[2]), nt[0],
+        nt[1], nt[2], tiles);
+    return cudaGetLastError();
+}
+
 // The mask as rows of 32 cells along x (vrc_cellmask_get): word (c'_z (ny + 1) + c'_y) cwx +
 // c'_x / 32, bit c'_x % 32, c' = c + 1. One thread per word.
 __global__ void cellmask_rows_kernel(const uint32_t *__restrict__ cells, int nx, int ny, int nz,

@@ -709,6 +709,10 @@ size_t cellmask_bytes(const int n[3]);
 cudaError_t launch_cellmask(const VolView &v, int B, const int nb[3], const uint8_t *occ,
                             const uint8_t *zrun_dev, float lo, float du, uint32_t *cells,
                             cudaStream_t st);
+// Occupancy bytes of the 8^3 tiles (cells 8t .. 8t + 7 per axis, tile 0 also the cells -1; nt =
+// ceil(n / 8) of them): 1 where the mask has an open cell.
+cudaError_t launch_tile_occupancy(const uint32_t *cells, const int n[3], const int nt[3],
+                                  uint8_t *tiles, cudaStream_t st);
 // The mask as rows of 32-cell words along x, the layout vrc_cellmask_get returns.
 long cellmask_row_words(const int n[3]);
 cudaError_t launch_cellmask_rows(const uint32_t *cells, const int n[3], uint32_t *out,
