@@ -726,6 +726,41 @@ __global__ void __launch_bounds__(256) dist_axis_kernel(const uint8_t *__restric
     }
 }
 
+// The same for rows of a multiple of 4 bricks, 4 bricks of a row a thread, as the byte pairs (0,
+// 2) and (1, 3) in 16-bit halves.
+template <int NIN>
+__global__ void __launch_bounds__(256) dist_axis4_kernel(const uint32_t *__restrict__ in,
+                                                         unsigned n4, unsigned len,
+                                                         unsigned stride4,
+                                                         uint32_t *__restrict__ out) {
+    constexpr int U = 8;  // loads in flight
+    const int h = blockIdx.y / NIN;
+    const uint32_t *f = in + (size_t)(blockIdx.y % NIN) * n4;
+    uint32_t *o = out + (size_t)blockIdx.y * n4;
+    const int s = h ? -(int)stride4 : (int)stride4;
+    for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n4; i += gridDim.x * 256u) {
+        const uint32_t *p = f + i;
+        const int pos = (int)((i / stride4) % len);
+        const int room = h ? pos : (int)len - 1 - pos;
+        const uint32_t w = p[0];
+        uint32_t b0 = w & 0x00ff00ffu, b1 = (w >> 8) & 0x00ff00ffu;
+        for (int d = 1; d <= room; d += U) {
+            const uint32_t m = __vmaxu2(b0, b1);
+            if ((int)max(m & 0xffffu, m >> 16) <= d) break;
+            uint32_t g[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) g[k] = p[(long)min(d + k, room) * s];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const uint32_t dd = (uint32_t)(d + k) * 0x10001u;
+                b0 = __vminu2(b0, __vmaxu2(dd, g[k] & 0x00ff00ffu));
+                b1 = __vminu2(b1, __vmaxu2(dd, (g[k] >> 8) & 0x00ff00ffu));
+            }
+        }
+        o[i] = b0 | (b1 << 8);
+    }
+}
+
 size_t box_dist_scratch_bytes(const int nb[3]) {
     return (size_t)(nb[0] + 1) * (nb[1] + 1) * (nb[2] + 1) * sizeof(int);
 }
@@ -735,13 +770,22 @@ size_t box_dist_scratch_bytes(const int nb[3]) {
 cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], int *scratch, uint8_t *dist,
                              cudaStream_t st) {
     const long n = (long)nb[0] * nb[1] * nb[2], rows = (long)nb[1] * nb[2];
-    const unsigned blocks = (unsigned)((n + 255) / 256 > 152L * 64 ? 152L * 64 : (n + 255) / 256);
     uint8_t *yf = (uint8_t *)scratch;
     dist_x_kernel<<<(unsigned)((rows + DX_WARPS - 1) / DX_WARPS), 32 * DX_WARPS, 0, st>>>(
         occ, nb[0], rows, dist);
-    dist_axis_kernel<2><<<dim3(blocks, 4), 256, 0, st>>>(dist, (unsigned)n, nb[1], nb[0], yf);
-    dist_axis_kernel<4><<<dim3(blocks, 8), 256, 0, st>>>(yf, (unsigned)n, nb[2], nb[0] * nb[1],
-                                                         dist);
+    auto blocks = [](long k) { return (unsigned)((k + 255) / 256 > 152L * 64 ? 152L * 64
+                                                                             : (k + 255) / 256); };
+    if (nb[0] % 4 == 0) {
+        const unsigned n4 = (unsigned)(n / 4), sy = nb[0] / 4, sz = sy * nb[1];
+        dist_axis4_kernel<2><<<dim3(blocks(n4), 4), 256, 0, st>>>((const uint32_t *)dist, n4, nb[1],
+                                                                  sy, (uint32_t *)yf);
+        dist_axis4_kernel<4><<<dim3(blocks(n4), 8), 256, 0, st>>>((const uint32_t *)yf, n4, nb[2],
+                                                                  sz, (uint32_t *)dist);
+        return cudaGetLastError();
+    }
+    dist_axis_kernel<2><<<dim3(blocks(n), 4), 256, 0, st>>>(dist, (unsigned)n, nb[1], nb[0], yf);
+    dist_axis_kernel<4><<<dim3(blocks(n), 8), 256, 0, st>>>(yf, (unsigned)n, nb[2], nb[0] * nb[1],
+                                                            dist);
     return cudaGetLastError();
 }
 
