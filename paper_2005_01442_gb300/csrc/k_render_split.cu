@@ -11,8 +11,8 @@
 //    in an occupied brick are written out, the others are appended to a queue with their
 //    colour and transmittance so far and the index of that sample;
 // 2. a grid sized to fill the device drains the queue, each group of SPLIT_G lanes claiming
-//    one ray at a time and finishing it with group_march (k_group.cuh): blocks of SPLIT_G
-//    consecutive samples composited by a scan of the "over" operator.
+//    one ray at a time and finishing it in blocks of SPLIT_G consecutive samples (march_block,
+//    k_group.cuh) composited by a scan of the "over" operator.
 //
 // Each ray is composited in the same order whatever the other rays do, and with the same
 // result with and without skipping (the hand-over index is fixed and blocks are aligned to
@@ -27,9 +27,10 @@ __global__ void __launch_bounds__(32 * SPLIT_RAY_WARPS, 16 / SPLIT_RAY_WARPS)
     split_head_body<ESL, CKPT>(L);
 }
 
-// Four CTAs per SM (64 registers, a few spills): the march is bound by the latency of
-// dependent loads, and 32 resident warps hide it better than 24 at 80 registers (measured:
-// 0.377 vs 0.392 ms per 1024^2 CT frame; five CTAs at 48 registers spill too much).
+// Four CTAs per SM (64 registers, a few spills): 32 resident warps hide the latency of dependent
+// loads better than 24 at 80 registers (a 1024^2 frame of a 256^3 CT / with soft tissue: 438 /
+// 1290 us against 448 / 1311, with 16 at 128 registers 533 / 1515, with 40 at 48 registers, which
+// spill, 461 / 1460).
 template <bool ESL, int MODE, bool CKPT, int PACKED>
 __global__ void __launch_bounds__(32 * SPLIT_WARPS, 4) split_tail_kernel(RenderLaunch L) {
     split_tail_body<ESL, MODE, CKPT, PACKED>(L);

@@ -84,12 +84,12 @@ __global__ void __launch_bounds__(WC_RAYS, 2) render_warp_kernel(RenderLaunch L)
         ray_float(rp, Pf, df, inv_df);
         const uint8_t *dist = nullptr;
         if (ESL) dist = L.dist + octant_of(df) * nbricks;
-        float RC0 = 0.0f, RC1 = 0.0f, RC2 = 0.0f, RT = 1.0f;
-        unsigned ex = 0;
+        March m = {0.0f, 0.0f, 0.0f, 1.0f, 0u, 0u};
         group_march<ESL, G>(L, rp, dist, Pf, df, inv_df, inv_step, s_rec[qi].j0, gmask, q, gbase,
-                            RC0, RC1, RC2, RT, ex, resampled);
-        executed += ex;
-        if (q == 0) L.out[pix] = make_float4(RC0, RC1, RC2, 1.0f - RT);
+                            m);
+        executed += m.executed;
+        resampled += m.resampled;
+        if (q == 0) L.out[pix] = make_float4(m.C0, m.C1, m.C2, 1.0f - m.T);
     }
 
     if (L.counters) {

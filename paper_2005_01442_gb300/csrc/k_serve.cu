@@ -100,19 +100,17 @@ __device__ __forceinline__ void serve_rays_body(const RenderLaunch &L, unsigned 
     const unsigned gmask = ((1u << SPLIT_G) - 1u) << gbase;
     const float inv_step = 1.0f / L.grid.step;
     const long nbricks = ESL ? (long)L.bricks.nb[0] * L.bricks.nb[1] * L.bricks.nb[2] : 0;
-    unsigned executed = 0, resampled = 0;
     for (unsigned c = c0 + group; c < c0 + chunk; c += 2) {
         const unsigned qi = c < nf ? c : L.split.cap - 1u - (c - nf);
         RayPos rp;
         int jlo, pix;
-        float RC0, RC1, RC2, RT;
-        split_load(L.split.rec + (long)qi * SPLIT_REC, rp, jlo, pix, RC0, RC1, RC2, RT);
+        March m = {};
+        split_load(L.split.rec + (long)qi * SPLIT_REC, rp, jlo, pix, m.C0, m.C1, m.C2, m.T);
         float Pf[3], df[3], inv_df[3];
         ray_float(rp, Pf, df, inv_df);
         const uint8_t *dist = ESL ? L.dist + octant_of(df) * nbricks : nullptr;
-        group_march<ESL, SPLIT_G>(L, rp, dist, Pf, df, inv_df, inv_step, jlo, gmask, q, gbase,
-                                  RC0, RC1, RC2, RT, executed, resampled);
-        if (q == 0) L.out[pix] = make_float4(RC0, RC1, RC2, 1.0f - RT);
+        group_march<ESL, SPLIT_G>(L, rp, dist, Pf, df, inv_df, inv_step, jlo, gmask, q, gbase, m);
+        if (q == 0) L.out[pix] = make_float4(m.C0, m.C1, m.C2, 1.0f - m.T);
     }
 }
 

@@ -95,12 +95,18 @@ __device__ __forceinline__ int leap_float(const BrickView &bv, const uint8_t *__
     const float margin = bv.margin;
     if (j >= nseg - 1) return j;  // the last segment's midpoint is not (j + 1/2) ds
     const float m = ((float)j + 0.5f) * step;
-    float pa[3];
+    const float B = float_small(bv.B), inv_B = bv.shift == 4 ? 0.0625f : 0.125f;
     int b[3];
+    float lo[3];
+    bool near = false;  // sample j must sit the margin inside its own brick (interior faces only)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        pa[k] = fmaf(m, df[k], Pf[k]);
-        b[k] = min(max((int)floorf(pa[k]), 0) >> bv.shift, bv.nb[k] - 1);
+        const float pa = fmaf(m, df[k], Pf[k]);
+        floor_small(pa * inv_B, b[k]);
+        b[k] = min(max(b[k], 0), bv.nb[k] - 1);
+        lo[k] = float_small(b[k]) * B;  // exact
+        const float in = pa - lo[k];
+        near |= (in < margin && b[k] > 0) || (in > B - margin && b[k] < bv.nb[k] - 1);
     }
     const int lin = (b[2] * bv.nb[1] + b[1]) * bv.nb[0] + b[0];
     if (lin != cache_lin) {
@@ -108,27 +114,16 @@ __device__ __forceinline__ int leap_float(const BrickView &bv, const uint8_t *__
         cache_r = dist[lin];
     }
     const int r = cache_r;
-    if (r == 0) return j;
+    if (r == 0 || near) return j;
+    // exit of the empty forward box of extent r - 1 bricks, faces moved inward by the margin
+    const float ahead = float_small(r) * B - margin;
     float texit = INFINITY;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        // sample j must sit the margin inside its own brick (interior faces only)
-        const float lo = (float)(b[k] * bv.B), hi = lo + (float)bv.B;
-        if ((b[k] > 0 && pa[k] < lo + margin) ||
-            (b[k] < bv.nb[k] - 1 && pa[k] > hi - margin))
-            return j;
-        // exit of the empty forward box of extent r - 1 bricks, face moved inward by the margin
-        float face;
-        if (df[k] > 0.0f) {
-            if (b[k] + r >= bv.nb[k]) continue;
-            face = (float)((b[k] + r) * bv.B) - margin;
-        } else if (df[k] < 0.0f) {
-            if (b[k] - r + 1 <= 0) continue;
-            face = (float)((b[k] - r + 1) * bv.B) + margin;
-        } else {
-            continue;
-        }
-        texit = fminf(texit, (face - Pf[k]) * inv_df[k]);
+        const bool fwd = df[k] > 0.0f;
+        const bool inside = fwd ? b[k] + r < bv.nb[k] : (df[k] < 0.0f && b[k] - r + 1 > 0);
+        const float face = fwd ? lo[k] + ahead : lo[k] + B - ahead;
+        if (inside) texit = fminf(texit, (face - Pf[k]) * inv_df[k]);
     }
     if (!(texit < INFINITY)) return nseg;
     // first sample whose midpoint may reach the moved face
@@ -369,9 +364,9 @@ __device__ __forceinline__ Classified classify(const TfView &tf, float v) {
     Classified k;
     k.u_raw = (v - tf.lo) * tf.du;
     const float u = fminf(fmaxf(k.u_raw, 0.0f), 255.0f);
-    floor_small(u, k.i0);
+    const float fl = fminf(floor_small(u, k.i0), 254.0f);
     k.i0 = min(k.i0, 254);
-    k.fu = u - (float)k.i0;
+    k.fu = u - fl;
     f32x2 e[4];
     load32(tf.tab + 2 * k.i0, e);
     const float2 dxy = unpack2(e[2]), dzw = unpack2(e[3]);
@@ -648,13 +643,21 @@ inline int ckpt_segments(const int n[3], float step, int seg) {
 VRC_HD int cell_blocks(int n) { return ((n + 3) >> 2) + 1; }
 VRC_HD int cell_tiles(int n) { return ((n + 7) >> 3) + 1; }
 
-// Bit of the cell holding sample base ip (ip in [-1, n-1]); 0: the sample's opacity is zero.
-__device__ __forceinline__ bool cell_open(const uint32_t *__restrict__ cells, const int n[3],
-                                          const int ip[3]) {
+// The word and the bit in it of the cell holding sample base ip (ip in [-1, n-1]).
+__device__ __forceinline__ uint32_t cell_word(const uint32_t *__restrict__ cells, const int n[3],
+                                              const int ip[3]) {
     const int cx = ip[0] + 4, cy = ip[1] + 4, cz = ip[2] + 4;
     const int blk = ((cz >> 2) * cell_blocks(n[1]) + (cy >> 2)) * cell_blocks(n[0]) + (cx >> 2);
-    const uint32_t w = __ldg(cells + 2 * blk + ((cz >> 1) & 1));
-    return (w >> (((cz & 1) << 4) | ((cy & 3) << 2) | (cx & 3))) & 1u;
+    return __ldg(cells + 2 * blk + ((cz >> 1) & 1));
+}
+__device__ __forceinline__ bool cell_bit(uint32_t w, const int ip[3]) {
+    return (w >> (((ip[2] & 1) << 4) | ((ip[1] & 3) << 2) | (ip[0] & 3))) & 1u;
+}
+
+// 0: the opacity of samples at base ip is zero.
+__device__ __forceinline__ bool cell_open(const uint32_t *__restrict__ cells, const int n[3],
+                                          const int ip[3]) {
+    return cell_bit(cell_word(cells, n, ip), ip);
 }
 
 // Quick skip test of sample j < nseg - 1 from its float position (the leap path's, within a
