@@ -32,7 +32,7 @@
 // on average, at 192 G/s measured: 36 a sample), and eight shared-memory atomics a sample
 // contended for the few table entries in use. Consecutive samples half a voxel apart share most
 // of their taps, so a box of 16 gives some 4.9 atomic sectors a sample instead. 256^3 float32 at
-// 512^2, soft tissue visible (17 M samples): 1.92 ms a view against 4.0 ms. What bounds it now is
+// 512^2, soft tissue visible (17 M samples): 1.80 ms a view against 4.0 ms. What bounds it now is
 // the chain of a warp's adds and the registers (16 warps an SM): 54% of the issue slots, 61% of
 // the L1 and shared-memory data path.
 #include "vrc_internal.h"
@@ -153,8 +153,12 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunc
         const float *ck_row = L.ckpt + (long)s_ray[qi].pix * L.ckpt_K;
         // what lies behind the current block: normalised colour and transmittance
         float cS0 = 0.0f, cS1 = 0.0f, cS2 = 0.0f, cU = 1.0f;
-        for (int k = min(jlast / seg, L.ckpt_K - 1); k >= k0; --k) {
-            const float Tk = ck_row[k];
+        const int klast = min(jlast / seg, L.ckpt_K - 1);
+        float ck = -1.0f;  // 32 segments' checkpoints at a time, one a lane
+        for (int k = klast; k >= k0; --k) {
+            const int back = (klast - k) & 31;
+            if (back == 0) ck = k - lane >= k0 ? ck_row[k - lane] : -1.0f;
+            const float Tk = __shfl_sync(0xffffffffu, ck, back);
             if (!(Tk >= 0.0f)) continue;  // no composited sample in this segment
             const int j1 = min(k * seg + seg, jlast + 1);
             int chunk = ADJ_CHUNK;
@@ -163,18 +167,26 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunc
             float f[NB][3], sv[NB], Tj[NB];
             unsigned live_bits[NB];
             float T = Tk;
+            uint32_t word[NB];
+            uint8_t empty[NB];
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {  // the blocks' look-ups in flight together
+                float delta;
+                const int j = min(k * seg + 32 * b + lane, rp.nseg - 1);
+                place(rp, step, L.grid.n, j, ip[b], f[b], delta);
+                if (ESL) {
+                    empty[b] = dist[brick_of(L.bricks, ip[b])];
+                    word[b] = L.cells ? cell_word(L.cells, L.grid.n, ip[b]) : 0xffffffffu;
+                }
+            }
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 const int j = k * seg + 32 * b + lane;
                 bool live = j < j1;
-                float delta, eT = 1.0f;
+                if (ESL) live = live && empty[b] == 0 && cell_bit(word[b], ip[b]);
+                const float delta = j < rp.nseg - 1 ? step : rp.dlast;
+                float eT = 1.0f;
                 sv[b] = 0.0f;
-                if (live) {
-                    place(rp, step, L.grid.n, j, ip[b], f[b], delta);
-                    if (ESL && (dist[brick_of(L.bricks, ip[b])] != 0 ||
-                                (L.cells && !cell_open(L.cells, L.grid.n, ip[b]))))
-                        live = false;
-                }
                 if (live) {
                     sv[b] = tricubic_rep(L.rep, ip[b], f[b]);
                     eT = 1.0f - segment_alpha(classify(L.tf, sv[b]).c.w, delta);
@@ -245,7 +257,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunc
                 const float a = fminf(fmaxf(c.c.w, 0.0f), ALPHA_MAX);
                 const bool up = c.c.w > 0.0f || (A.open_alpha && c.c.w == 0.0f);
                 const float da = (up && c.c.w <= ALPHA_MAX)
-                                     ? delta * exp2f((delta - 1.0f) * __log2f(1.0f - a))
+                                     ? delta * ex2((delta - 1.0f) * lg2(1.0f - a))
                                      : 0.0f;
                 const float d_a = dalpha * da;
                 float ds = 0.0f;
