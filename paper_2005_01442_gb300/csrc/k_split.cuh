@@ -63,9 +63,17 @@ __device__ __forceinline__ void split_tail_body(const RenderLaunch &L) {
     CkState ck = {};
     while (true) {
         if (!__any_sync(FULL, has)) {
+            // two rays; the last warp to find none left leaves the queue empty for the next render
             unsigned c = 0;
-            if (q == 0) c = atomicAdd(&L.split.head[1], 1u);
-            c = __shfl_sync(FULL, c, gbase);
+            if (lane == 0) c = atomicAdd(&L.split.head[1], 2u);
+            c = __shfl_sync(FULL, c, 0);
+            if (c >= total) {
+                const unsigned warps = gridDim.x * (blockDim.x >> 5);
+                if (lane == 0 && c == ((total + 1u) & ~1u) + 2u * (warps - 1u))
+                    L.split.head[0] = L.split.head[1] = L.split.head[2] = 0u;
+                break;
+            }
+            c += lane / G;
             has = c < total;
             if (has) {
                 const unsigned qi = c < nf ? c : L.split.cap - 1u - (c - nf);
@@ -91,7 +99,6 @@ __device__ __forceinline__ void split_tail_body(const RenderLaunch &L) {
                 }
             }
             __syncwarp();
-            if (!__any_sync(FULL, has)) break;
         }
         const float df[3] = {rp.d[0].hi, rp.d[1].hi, rp.d[2].hi};
         if (ESL) {

@@ -77,6 +77,7 @@ int lanes_of(int kernel) { return kernel == 3 ? 4 : kernel == 4 ? 8 : kernel == 
 // in order, so they can share it): a 256-byte header (pushed, claimed counts), then `cap`
 // ray records of SPLIT_REC float4.
 struct SplitBuf {
+    bool clear = false;  // the counters must be set to zero before the next render
     unsigned char *base = nullptr;
     size_t cap = 0;
 };
@@ -642,6 +643,18 @@ vrc_status split_queue(vrc_ctx *ctx, cudaStream_t st, size_t need, RaySplit &q) 
         const size_t bytes = 256 + need * SPLIT_REC * sizeof(float4);
         CK(cudaMalloc(&b.base, bytes), "cudaMalloc(split queue)");
         b.cap = need;
+        b.clear = true;
+    }
+    if (b.clear) {
+        // on a stream of its own, so that it happens now even if st is being captured (nothing
+        // uses a new queue, and after a failed launch nothing does)
+        cudaStream_t own;
+        CK(cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking), "cudaStreamCreate");
+        cudaError_t e = cudaMemsetAsync(b.base, 0, 3 * sizeof(unsigned), own);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(own);
+        cudaStreamDestroy(own);
+        CK(e, "split queue reset");
+        b.clear = false;
     }
     q.head = (unsigned *)b.base;
     q.rec = (float4 *)(b.base + 256);
@@ -698,8 +711,13 @@ vrc_status launch_render(vrc_ctx *ctx, const vrc_params *params, RenderLaunch &L
         // were slower)
         L.split.long_len = (unsigned)(0.35f * (L.grid.n[0] + L.grid.n[1] + L.grid.n[2]) / 3.0f /
                                       L.grid.step);
-        CK(cudaMemsetAsync(L.split.head, 0, 3 * sizeof(unsigned), st), "split queue reset");
-        CK(launch_render_split(L, st), "render launch");
+        // the queue is empty: cleared when it was made and by the end of each second phase
+        const cudaError_t e = launch_render_split(L, st);
+        if (e != cudaSuccess) {
+            cudaStreamSynchronize(st);
+            ctx->split[st].clear = true;
+            return cuda_fail(ctx, e, "render launch");
+        }
     } else if (k >= 2 && k <= 5) {
         CK(launch_render_warp(L, lanes_of(k), st), "render launch");
     } else if (k == 7) {

@@ -755,7 +755,7 @@ size_t tma_map_bytes();
 cudaError_t encode_tma_map(void *map_out, const float *base, int pnx, int pny, int pnz);
 cudaError_t launch_render_tma(const void *map, const RenderLaunch &L, cudaStream_t st);
 cudaError_t launch_render_warp(const RenderLaunch &L, int lanes_per_ray, cudaStream_t st);
-// Both phases of the split render; L.split.head must be zero (it is left nonzero).
+// Both phases of the split render; L.split.head must be zero, and is again at the end.
 cudaError_t launch_render_split(const RenderLaunch &L, cudaStream_t st);
 
 // Reverse mode of one render: grad_out is the loss gradient per pixel (H x W x RGBA);
