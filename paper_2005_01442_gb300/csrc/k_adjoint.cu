@@ -392,9 +392,11 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunc
 
 template <int NB>
 static void launch_adjoint_n(const AdjointLaunch &A, cudaStream_t st) {
-    // a tile of 8 x 4 pixels a CTA, or 4 x 2 where 8 x 4 would leave SMs without one
+    // a tile of 8 x 4 pixels a CTA, or 4 x 4 where 8 x 4 would leave SMs without one; not fewer:
+    // every CTA adds its table sums to the same 1024 floats, whose error grows with the number of
+    // additions (4 x 2: 1.5 times the error of 4 x 4 for a 98 x 460 image)
     const long pixels = (long)A.L.cam.width * A.L.cam.height;
-    const int tw = pixels < 64 * 1024 ? 2 : 3, th = tw - 1;
+    const int tw = pixels < 64 * 1024 ? 2 : 3, th = 2;
     const unsigned grid = (unsigned)((((long)A.L.cam.width + (1 << tw) - 1) >> tw) *
                                      ((A.L.cam.height + (1 << th) - 1) >> th));
     const bool esl = A.L.dist != nullptr, vg = A.grad_vol != nullptr;
