@@ -7,8 +7,6 @@
 // integer decision "is any table opacity > 0 on the brick's value range", taken in float32.
 #include <string.h>
 
-#include <type_traits>
-
 #include "vrc_internal.h"
 
 namespace vrc {
@@ -181,6 +179,12 @@ struct Lim<int16_t> {
     __device__ static int16_t lo() { return -32768; }
     __device__ static int16_t hi() { return 32767; }
 };
+template <>
+struct Lim<float> {
+    __device__ static float lo() { return -INFINITY; }
+    __device__ static float hi() { return INFINITY; }
+};
+
 // Two 16-bit values at a time.
 template <typename T>
 __device__ __forceinline__ uint32_t min2(uint32_t a, uint32_t b) {
@@ -204,14 +208,13 @@ __device__ __forceinline__ T tmax(T a, T b) { return a > b ? a : b; }
 
 // Min/max over rows of brick bx's apron, x in [bx*B - 1, bx*B + B + 1]: the padded row's elements
 // bx*B + 1 .. bx*B + B + 3, i.e. the brick's own span but for its first element, and the first 4
-// elements of the next span. A lane takes the spans of one brick, 16 bytes a load, and keeps the
-// two extremes apart; the next lane's first-4 extreme is fetched once, after the last row. The
+// elements of the next span. 16-bit: a lane takes the span of one brick, 16 bytes a load, and keeps
+// the two extremes apart; the next lane's first-4 extreme is fetched once, after the last row. The
 // pad replicates the edge voxels (also in the rounding of pnx, a multiple of 8), so what lies
 // past a row's end adds nothing. 16-bit voxels are compared two at a time.
 template <typename T>
 struct Pair16 {  // 8 elements in 4 words
     using V = uint32_t;
-    static constexpr int N = 8;
     __device__ static V none_lo() { return (uint32_t)(uint16_t)Lim<T>::hi() * 0x10001u; }
     __device__ static V none_hi() { return (uint32_t)(uint16_t)Lim<T>::lo() * 0x10001u; }
     __device__ static V least(V a, V b) { return min2<T>(a, b); }
@@ -220,33 +223,44 @@ struct Pair16 {  // 8 elements in 4 words
     __device__ static T low(V a) { return tmin((T)a, (T)(a >> 16)); }
     __device__ static T high(V a) { return tmax((T)a, (T)(a >> 16)); }
 };
-struct Single32 {  // 4 elements in 4 words
-    using V = float;
-    static constexpr int N = 4;
-    __device__ static V none_lo() { return INFINITY; }
-    __device__ static V none_hi() { return -INFINITY; }
-    __device__ static V least(V a, V b) { return tmin(a, b); }
-    __device__ static V most(V a, V b) { return tmax(a, b); }
-    __device__ static float low(V a) { return a; }
-    __device__ static float high(V a) { return a; }
-};
+// The whole apron span of a row by one thread (float32).
+template <int B>
+__device__ __forceinline__ void apron_row(const float *__restrict__ r, int bx, int pnx, float &lo,
+                                          float &hi) {
+    float v[B + 4];
+    const int i0 = bx * B;
+    if (i0 + B + 4 <= pnx) {
+        const float4 *p = reinterpret_cast<const float4 *>(r + i0);
+#pragma unroll
+        for (int k = 0; k < (B + 4) / 4; ++k) {
+            const float4 w = __ldg(p + k);
+            memcpy(&v[k * 4], &w, 16);
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < B + 4; ++e) v[e] = r[min(i0 + e, pnx - 1)];
+    }
+#pragma unroll
+    for (int e = 1; e < B + 4; ++e) {
+        lo = tmin(lo, v[e]);
+        hi = tmax(hi, v[e]);
+    }
+}
 
 // One CTA per brick row (by, bz): thread x handles brick bx (64 at a time) and sweeps the
 // rows of the (y, z) apron, thread y interleaves those rows; partial min/max are combined
 // through shared memory. Each voxel is read from HBM about once (neighbouring rows of bricks
 // re-read the overlap through L2). Exact for every dtype.
 // Bound: latency of the loads. 512^2 x 400 int16, B = 8: 53 us (217 MB read, 4.1 TB/s); with three
-// 8-byte loads of the overlapping 12 elements a brick and row 82 us; 256^3 float32 35 -> 26 us.
+// 8-byte loads of the overlapping 12 elements a brick and row 82 us. Float32 spans are 32 bytes or
+// more and keep overlapping loads, row by row over the threads y: 36 us for 256^3 (41 us by the
+// lanes' own spans, 56 us slice by slice).
 constexpr int BM_TX = 64, BM_TY = 4;
 
 template <typename T, int B>
 __global__ void __launch_bounds__(BM_TX *BM_TY) brick_minmax_kernel(VolView v, int nbx, int nby,
                                                                      int nbz, T *__restrict__ mn,
                                                                      T *__restrict__ mx) {
-    using X = typename std::conditional<sizeof(T) == 2, Pair16<T>, Single32>::type;
-    using V = typename X::V;
-    constexpr int PIECES = B / X::N;      // 16-byte loads of a span
-    constexpr int HEAD = sizeof(T) == 2 ? 2 : 4;  // words that hold 4 elements
     __shared__ T s_lo[BM_TY][BM_TX], s_hi[BM_TY][BM_TX];
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int by = blockIdx.x % nby, bz = blockIdx.x / nby;
@@ -256,60 +270,63 @@ __global__ void __launch_bounds__(BM_TX *BM_TY) brick_minmax_kernel(VolView v, i
     const T *base = (const T *)v.base;
     for (int bx0 = 0; bx0 < nbx; bx0 += BM_TX) {
         const int bx = bx0 + tx;
-        V lo = X::none_lo(), hi = X::none_hi();    // own span without its first element
-        V flo = X::none_lo(), fhi = X::none_hi();  // first 4 elements of the span
-        V nlo = X::none_lo(), nhi = X::none_hi();  // lane 31: of the next lane's span
-        // spans (of whole 8-element pieces) inside the row; lanes past the last brick read theirs
-        // for the lane before
-        const bool last = (tx & 31) == 31 && (bx + 1) * B < v.pnx;
-        for (int z = z0 + ty; z <= z1; z += BM_TY) {
-            const T *row = base + ((long)(z + PAD) * v.pny + (y0 + PAD)) * v.pnx + bx * B;
-#pragma unroll 6
-            for (int y = y0; y <= y1; ++y, row += v.pnx) {
-#pragma unroll
-                for (int k = 0; k < PIECES; ++k) {
-                    if (bx * B + k * X::N >= v.pnx) break;
-                    V w[4];
-                    const uint4 q = __ldg(reinterpret_cast<const uint4 *>(row) + k);
-                    memcpy(w, &q, 16);
-                    if (k == 0) {
-#pragma unroll
-                        for (int i = 0; i < HEAD; ++i) {
-                            flo = X::least(flo, w[i]);
-                            fhi = X::most(fhi, w[i]);
-                        }
-                        if constexpr (sizeof(T) == 2) w[0] = X::skip_first(w[0]);
-                        else w[0] = w[1];
-                    }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        lo = X::least(lo, w[i]);
-                        hi = X::most(hi, w[i]);
-                    }
+        T least = Lim<T>::hi(), most = Lim<T>::lo();
+        if constexpr (sizeof(T) == 4) {
+            if (bx < nbx) {
+                const int wy = y1 - y0 + 1, rows = wy * (z1 - z0 + 1);
+                for (int r = ty; r < rows; r += BM_TY) {
+                    const int y = y0 + r % wy, z = z0 + r / wy;
+                    apron_row<B>(base + ((long)(z + PAD) * v.pny + (y + PAD)) * v.pnx, bx, v.pnx,
+                                 least, most);
                 }
-                if (last) {
-                    V w[4];
-                    if constexpr (sizeof(T) == 2) {
-                        const uint2 q = __ldg(reinterpret_cast<const uint2 *>(row + B));
-                        memcpy(w, &q, 8);
-                    } else {
-                        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(row + B));
-                        memcpy(w, &q, 16);
-                    }
+            }
+        } else {
+            using X = Pair16<T>;
+            using V = typename X::V;
+            V lo = X::none_lo(), hi = X::none_hi();    // own span without its first element
+            V flo = X::none_lo(), fhi = X::none_hi();  // first 4 elements of the span
+            V nlo = X::none_lo(), nhi = X::none_hi();  // lane 31: of the next lane's span
+            // spans (of whole 8-element pieces) inside the row; lanes past the last brick read
+            // theirs for the lane before
+            const bool last = (tx & 31) == 31 && (bx + 1) * B < v.pnx;
+            for (int z = z0 + ty; z <= z1; z += BM_TY) {
+                const T *row = base + ((long)(z + PAD) * v.pny + (y0 + PAD)) * v.pnx + bx * B;
+#pragma unroll 6
+                for (int y = y0; y <= y1; ++y, row += v.pnx) {
 #pragma unroll
-                    for (int i = 0; i < HEAD; ++i) {
-                        nlo = X::least(nlo, w[i]);
-                        nhi = X::most(nhi, w[i]);
+                    for (int k = 0; k < B / 8; ++k) {
+                        if (bx * B + k * 8 >= v.pnx) break;
+                        V w[4];
+                        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(row) + k);
+                        memcpy(w, &q, 16);
+                        if (k == 0) {
+#pragma unroll
+                            for (int i = 0; i < 2; ++i) {
+                                flo = X::least(flo, w[i]);
+                                fhi = X::most(fhi, w[i]);
+                            }
+                            w[0] = X::skip_first(w[0]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            lo = X::least(lo, w[i]);
+                            hi = X::most(hi, w[i]);
+                        }
+                    }
+                    if (last) {
+                        const uint2 q = __ldg(reinterpret_cast<const uint2 *>(row + B));
+                        nlo = X::least(nlo, X::least(q.x, q.y));
+                        nhi = X::most(nhi, X::most(q.x, q.y));
                     }
                 }
             }
+            const V dlo = __shfl_down_sync(0xffffffffu, flo, 1);
+            const V dhi = __shfl_down_sync(0xffffffffu, fhi, 1);
+            least = X::low(X::least(lo, (tx & 31) == 31 ? nlo : dlo));
+            most = X::high(X::most(hi, (tx & 31) == 31 ? nhi : dhi));
         }
-        const V dlo = __shfl_down_sync(0xffffffffu, flo, 1);
-        const V dhi = __shfl_down_sync(0xffffffffu, fhi, 1);
-        lo = X::least(lo, (tx & 31) == 31 ? nlo : dlo);
-        hi = X::most(hi, (tx & 31) == 31 ? nhi : dhi);
-        s_lo[ty][tx] = X::low(lo);
-        s_hi[ty][tx] = X::high(hi);
+        s_lo[ty][tx] = least;
+        s_hi[ty][tx] = most;
         __syncthreads();
         if (ty == 0 && bx < nbx) {
             T l = s_lo[0][tx], h = s_hi[0][tx];
