@@ -511,9 +511,9 @@ def main():
             "fp32_sgemm_tflops_measured": sgemm,
             "other_workloads_and_kernels": legs,
             "cpu_baseline": cpu, "e2e": e2e,
-            # bricks, occupancy, 3 summed-volume passes, distance, cell mask; per frame the
+            # bricks, occupancy, 3 distance passes, cell mask; per frame the
             # split render's two kernels (one for the per-ray kernel)
-            "gpu_launches": args.steps * (7 + args.cameras * (2 if args.kernel in (0, 6) else 1)),
+            "gpu_launches": args.steps * (6 + args.cameras * (2 if args.kernel in (0, 6) else 1)),
             "clocks": clocks,
         }
         if not args.no_serve:
