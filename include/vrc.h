@@ -88,7 +88,10 @@ typedef struct {
  *                  6 = split render: one lane per ray sets the ray up and leaps to its
  *                  first sample in an occupied brick, then groups of 16 lanes drawn from the
  *                  whole device finish the queued rays (the context keeps a queue of 112
- *                  bytes per pixel for each stream it renders on).
+ *                  bytes per pixel for each stream it renders on, and one more for renders
+ *                  captured on that stream: a graph may be replayed while the stream renders,
+ *                  but graphs captured on one stream must not be replayed at the same time.
+ *                  A stream must have rendered an image of that size before the capture).
  *                  All kernels compute the same method; images agree within float
  *                  rounding of the compositing order. Other values: VRC_ERR_ARG.
  *   interp         0 = uniform cubic B-spline (64 taps, the paper's choice), 1 = trilinear

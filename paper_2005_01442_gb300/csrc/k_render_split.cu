@@ -34,6 +34,9 @@ __global__ void __launch_bounds__(32 * SPLIT_RAY_WARPS, 16 / SPLIT_RAY_WARPS)
 template <bool ESL, int MODE, bool CKPT, int PACKED>
 __global__ void __launch_bounds__(32 * SPLIT_WARPS, 4) split_tail_kernel(RenderLaunch L) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    // The counters of the stream's next render: the render before this one, which used them, has
+    // ended, and the next one starts after this one. Whatever they hold, each frame starts clean.
+    if (L.split.next && blockIdx.x == 0 && threadIdx.x < 3) L.split.next[threadIdx.x] = 0u;
     split_tail_body<ESL, MODE, CKPT, PACKED>(L);
 }
 

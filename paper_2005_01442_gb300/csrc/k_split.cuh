@@ -63,16 +63,10 @@ __device__ __forceinline__ void split_tail_body(const RenderLaunch &L) {
     CkState ck = {};
     while (true) {
         if (!__any_sync(FULL, has)) {
-            // two rays; the last warp to find none left leaves the queue empty for the next render
             unsigned c = 0;
-            if (lane == 0) c = atomicAdd(&L.split.head[1], 2u);
+            if (lane == 0) c = atomicAdd(&L.split.head[1], 2u);  // two rays
             c = __shfl_sync(FULL, c, 0);
-            if (c >= total) {
-                const unsigned warps = gridDim.x * (blockDim.x >> 5);
-                if (lane == 0 && c == ((total + 1u) & ~1u) + 2u * (warps - 1u))
-                    L.split.head[0] = L.split.head[1] = L.split.head[2] = 0u;
-                break;
-            }
+            if (c >= total) break;
             c += lane / G;
             has = c < total;
             if (has) {

@@ -74,12 +74,23 @@ int slot_of(int B) { return B == 16 ? 1 : 0; }
 int lanes_of(int kernel) { return kernel == 3 ? 4 : kernel == 4 ? 8 : kernel == 5 ? 16 : 32; }
 
 // Queue of the split render, one per stream that renders with it (renders on one stream run
-// in order, so they can share it): a 256-byte header (pushed, claimed counts), then `cap`
-// ray records of SPLIT_REC float4.
+// in order, so they can share it): a 256-byte header (two sets of counters, used in turn: a
+// render clears the other set for the one after it), then `cap` ray records of SPLIT_REC float4.
 struct SplitBuf {
-    bool clear = false;  // the counters must be set to zero before the next render
     unsigned char *base = nullptr;
     size_t cap = 0;
+    unsigned turn = 0;   // the set of the next render
+    bool clear = false;  // both sets must be set to zero before the next render
+};
+
+// Renders captured on a stream have a queue of their own, since their graph may be replayed
+// while the stream renders. Each clears its counters by a node of the graph. A queue that grew
+// too small for a later capture stays for the graphs that use it (sizes at least double, so
+// those together hold less than the one in use).
+struct CaptureBuf {
+    unsigned char *base = nullptr;
+    size_t cap = 0;
+    std::vector<unsigned char *> old;
 };
 
 // Object-order decomposition of a volume into a grid of pieces of whole bricks, for one
@@ -120,6 +131,7 @@ struct vrc_ctx {
     float4 *host_img = nullptr;  // device image for vrc_render_host
     size_t host_img_bytes = 0;
     std::map<cudaStream_t, SplitBuf> split;  // split-render queues by stream
+    std::map<cudaStream_t, CaptureBuf> captured;  // and those of renders captured on a stream
     std::map<int, Plan> plans;               // piece grids (vrc_pieces_build)
     // vrc_render_host_batch: two device images, a copy stream and their events
     float4 *batch_img[2] = {nullptr, nullptr};
@@ -632,6 +644,33 @@ vrc_status prepare_render(vrc_ctx *ctx, int vol_id, int tf_id, const vrc_camera 
     return VRC_OK;
 }
 
+size_t queue_bytes(size_t records) { return 256 + records * SPLIT_REC * sizeof(float4); }
+
+// The queue of renders captured on stream st, grown to hold `need` records, and the node that
+// clears it.
+vrc_status capture_queue(vrc_ctx *ctx, cudaStream_t st, size_t need, RaySplit &q) {
+    CaptureBuf &b = ctx->captured[st];
+    if (b.cap < need) {
+        const size_t cap = std::max(need, 2 * b.cap);
+        unsigned char *base = nullptr;
+        // an allocation beside the capture, not a part of it
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode), "capture mode");
+        const cudaError_t e = cudaMalloc(&base, queue_bytes(cap));
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        CK(e, "cudaMalloc(split queue of captured renders)");
+        if (b.base) b.old.push_back(b.base);
+        b.base = base;
+        b.cap = cap;
+    }
+    q.head = (unsigned *)b.base;
+    q.next = nullptr;
+    q.rec = (float4 *)(b.base + 256);
+    q.cap = (unsigned)b.cap;
+    CK(cudaMemsetAsync(q.head, 0, 3 * sizeof(unsigned), st), "split queue reset");
+    return VRC_OK;
+}
+
 // The queue of the split render on stream st, grown to hold `need` records.
 vrc_status split_queue(vrc_ctx *ctx, cudaStream_t st, size_t need, RaySplit &q) {
     SplitBuf &b = ctx->split[st];
@@ -640,23 +679,25 @@ vrc_status split_queue(vrc_ctx *ctx, cudaStream_t st, size_t need, RaySplit &q) 
         cudaFree(b.base);
         b.base = nullptr;
         b.cap = 0;
-        const size_t bytes = 256 + need * SPLIT_REC * sizeof(float4);
-        CK(cudaMalloc(&b.base, bytes), "cudaMalloc(split queue)");
+        CK(cudaMalloc(&b.base, queue_bytes(need)), "cudaMalloc(split queue)");
         b.cap = need;
         b.clear = true;
     }
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(st, &capture), "capture status");
+    if (capture != cudaStreamCaptureStatusNone) return capture_queue(ctx, st, need, q);
     if (b.clear) {
-        // on a stream of its own, so that it happens now even if st is being captured (nothing
-        // uses a new queue, and after a failed launch nothing does)
+        // on a stream of its own
         cudaStream_t own;
         CK(cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking), "cudaStreamCreate");
-        cudaError_t e = cudaMemsetAsync(b.base, 0, 3 * sizeof(unsigned), own);
+        cudaError_t e = cudaMemsetAsync(b.base, 0, 256, own);
         if (e == cudaSuccess) e = cudaStreamSynchronize(own);
         cudaStreamDestroy(own);
         CK(e, "split queue reset");
         b.clear = false;
     }
-    q.head = (unsigned *)b.base;
+    q.head = (unsigned *)(b.base + 128 * b.turn);
+    q.next = (unsigned *)(b.base + 128 * (b.turn ^ 1));
     q.rec = (float4 *)(b.base + 256);
     q.cap = (unsigned)b.cap;
     return VRC_OK;
@@ -711,13 +752,17 @@ vrc_status launch_render(vrc_ctx *ctx, const vrc_params *params, RenderLaunch &L
         // were slower)
         L.split.long_len = (unsigned)(0.35f * (L.grid.n[0] + L.grid.n[1] + L.grid.n[2]) / 3.0f /
                                       L.grid.step);
-        // the queue is empty: cleared when it was made and by the end of each second phase
         const cudaError_t e = launch_render_split(L, st);
-        if (e != cudaSuccess) {
-            cudaStreamSynchronize(st);
-            ctx->split[st].clear = true;
-            return cuda_fail(ctx, e, "render launch");
+        if (L.split.next) {  // (a captured render's queue is cleared by its graph)
+            SplitBuf &b = ctx->split[st];
+            if (e == cudaSuccess) {
+                b.turn ^= 1;
+            } else {
+                cudaStreamSynchronize(st);
+                b.clear = true;
+            }
         }
+        CK(e, "render launch");
     } else if (k >= 2 && k <= 5) {
         CK(launch_render_warp(L, lanes_of(k), st), "render launch");
     } else if (k == 7) {
@@ -778,6 +823,10 @@ vrc_status vrc_destroy(vrc_ctx *ctx) {
     cudaFree(ctx->err_word);
     cudaFree(ctx->host_img);
     for (auto &kv : ctx->split) cudaFree(kv.second.base);
+    for (auto &kv : ctx->captured) {
+        cudaFree(kv.second.base);
+        for (unsigned char *b : kv.second.old) cudaFree(b);
+    }
     for (auto &kv : ctx->plans) free_plan(kv.second);
     for (int b = 0; b < 2; ++b) {
         cudaFree(ctx->batch_img[b]);

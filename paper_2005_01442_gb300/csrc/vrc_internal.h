@@ -542,6 +542,7 @@ constexpr int SPLIT_G = 16;
 constexpr int SPLIT_J0 = 0;  // a multiple of SPLIT_G
 struct RaySplit {
     unsigned *head;     // [records at the front, records claimed, records at the back]
+    unsigned *next;     // NULL, or the counters of the next render, which the second phase clears
     float4 *rec;        // SPLIT_REC float4 per queued ray (split_store)
     unsigned cap;       // records the queue holds (>= the image's pixels)
     unsigned long_len;  // rays with more samples left go to the front (claimed first)
@@ -755,7 +756,8 @@ size_t tma_map_bytes();
 cudaError_t encode_tma_map(void *map_out, const float *base, int pnx, int pny, int pnz);
 cudaError_t launch_render_tma(const void *map, const RenderLaunch &L, cudaStream_t st);
 cudaError_t launch_render_warp(const RenderLaunch &L, int lanes_per_ray, cudaStream_t st);
-// Both phases of the split render; L.split.head must be zero, and is again at the end.
+// Both phases of the split render; L.split.head must be zero. L.split.next, if given, is zero at
+// the end.
 cudaError_t launch_render_split(const RenderLaunch &L, cudaStream_t st);
 
 // Reverse mode of one render: grad_out is the loss gradient per pixel (H x W x RGBA);
