@@ -687,13 +687,7 @@ vrc_status split_queue(vrc_ctx *ctx, cudaStream_t st, size_t need, RaySplit &q) 
     CK(cudaStreamIsCapturing(st, &capture), "capture status");
     if (capture != cudaStreamCaptureStatusNone) return capture_queue(ctx, st, need, q);
     if (b.clear) {
-        // on a stream of its own
-        cudaStream_t own;
-        CK(cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking), "cudaStreamCreate");
-        cudaError_t e = cudaMemsetAsync(b.base, 0, 256, own);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(own);
-        cudaStreamDestroy(own);
-        CK(e, "split queue reset");
+        CK(cudaMemsetAsync(b.base, 0, 256, st), "split queue reset");
         b.clear = false;
     }
     q.head = (unsigned *)(b.base + 128 * b.turn);
@@ -755,12 +749,8 @@ vrc_status launch_render(vrc_ctx *ctx, const vrc_params *params, RenderLaunch &L
         const cudaError_t e = launch_render_split(L, st);
         if (L.split.next) {  // (a captured render's queue is cleared by its graph)
             SplitBuf &b = ctx->split[st];
-            if (e == cudaSuccess) {
-                b.turn ^= 1;
-            } else {
-                cudaStreamSynchronize(st);
-                b.clear = true;
-            }
+            if (e == cudaSuccess) b.turn ^= 1;
+            else b.clear = true;
         }
         CK(e, "render launch");
     } else if (k >= 2 && k <= 5) {
