@@ -18,9 +18,9 @@ namespace vrc {
 // L2), from where consecutive lanes write consecutive 32-byte pieces of the blocks, past L2 (the
 // padded copy, which the brick table reads next, may stay). Words of a row lie VL_Y and VL_Z
 // apart, so that the four rows read at once fall on different banks.
-// Bound: HBM, 2 (or 4) bytes read, as many padded and 16 (32) of render layout written per voxel.
+// Bound: HBM, 2 (or 4) bytes read, as many padded and 16 of render layout written per voxel.
 // 512^2 x 400 int16 (2.1 GB): 356 us, 5.9 TB/s; a warp per row that read its four source rows
-// element by element, which the L1 data path bound: 388 us. 256^3 float32 (0.67 GB): 119 us.
+// element by element, which the L1 data path bound: 388 us.
 constexpr int VL_WARPS = 8, VL_SPAN = 128, VL_Y = 136, VL_Z = 432;
 
 // 32 bytes to a 32-byte boundary, not kept in L2.
@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(32 * VL_WARPS)
     volume_layouts_kernel(const T *__restrict__ src, int nx, int ny, int nz, T *__restrict__ pad,
                           int pnx, char *__restrict__ rep, int rnx, int rny, int rnz) {
     constexpr int PER = 4 / (int)sizeof(T), SPAN = VL_SPAN * PER;  // voxels a word, a span
-    constexpr int ENTRY = sizeof(T) == 2 ? 16 : 32;
+    constexpr int BLOCK = 8 * ENTRY_BYTES;
     __shared__ __align__(16) uint32_t s_rows[VL_WARPS][3 * VL_Z];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *rows = s_rows[warp];
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(32 * VL_WARPS)
     }
     const bool words = (low & 3) == 0;  // 16-bit voxels 2i, 2i + 1 in one load
     const bool blocks = by < rny && bz < rnz;
-    char *out = rep + ((size_t)bz * rny + by) * rnx * 8 * ENTRY;
+    char *out = rep + ((size_t)bz * rny + by) * rnx * BLOCK;
     for (int x0 = 0; x0 < max(pnx, 2 * rnx); x0 += SPAN) {
         __syncwarp();  // the span before has been read
         // padded elements x0 .. x0 + SPAN + 3
@@ -89,13 +89,13 @@ __global__ void __launch_bounds__(32 * VL_WARPS)
         }
         if (!blocks) continue;
         const int kend = min(rnx - x0 / 2, SPAN / 2);
+        // lane: the entries x' = 2k, 2k + 1 of (y', z') = (2 by + g, 2 bz + h) in block k
+        const int g = lane & 1, h = (lane >> 1) & 1;
+        const uint32_t *s0 = rows + g * VL_Y + h * VL_Z;
+        char *to = out + (size_t)(x0 / 2) * BLOCK + 2 * ENTRY_BYTES * (lane & 3);
         if constexpr (sizeof(T) == 2) {
-            // lane: the entries x' = 2k, 2k + 1 of (y', z') = (2 by + g, 2 bz + h) in block k
-            const int g = lane & 1, h = (lane >> 1) & 1;
-            const uint32_t *s0 = rows + g * VL_Y + h * VL_Z;
             // int16: bias 32768, i.e. the sign bit flipped
             const uint32_t flip = (T)-1 < (T)0 ? 0x80008000u : 0u;
-            char *to = out + (size_t)(x0 / 2) * 8 * ENTRY + 32 * (lane & 3);
             for (int k = lane >> 2; k < kend; k += 8) {
                 uint32_t e[3][2];  // pairs of voxel 2k - 2 + i of row y
 #pragma unroll
@@ -107,18 +107,13 @@ __global__ void __launch_bounds__(32 * VL_WARPS)
                 }
                 const uint32_t v[8] = {e[0][0], e[1][0], e[0][1], e[1][1],
                                        e[1][0], e[2][0], e[1][1], e[2][1]};
-                store32_streaming(to + k * (8 * ENTRY), v);
+                store32_streaming(to + k * BLOCK, v);
             }
         } else {
-            // lane: the entry of slot lane & 7 in block k
-            const int g = (lane >> 1) & 1, h = (lane >> 2) & 1;
-            const uint32_t *s0 = rows + g * VL_Y + h * VL_Z + (lane & 1);
-            char *to = out + (size_t)(x0 / 2) * 8 * ENTRY + ENTRY * (lane & 7);
-            for (int k = lane >> 3; k < kend; k += 4) {
+            for (int k = lane >> 2; k < kend; k += 8) {
                 const uint32_t *a = s0 + 2 * k, *b = a + VL_Z;
-                const uint32_t v[8] = {a[0], b[0], a[1], b[1],
-                                       a[VL_Y], b[VL_Y], a[VL_Y + 1], b[VL_Y + 1]};
-                store32_streaming(to + k * (8 * ENTRY), v);
+                const uint32_t v[8] = {a[0], b[0], a[1], b[1], a[1], b[1], a[2], b[2]};
+                store32_streaming(to + k * BLOCK, v);
             }
         }
     }
@@ -129,8 +124,8 @@ ReplView rep_view(const void *base, int dtype, const int n[3]) {
     r.base = base;
     r.packed = dtype != DT_F32;
     r.rnx = (n[0] + 4) / 2;
-    r.rny = (n[1] + 4) / 2;
-    r.row = (r.packed ? 128 : 256) * (size_t)r.rnx;
+    r.rny = (n[1] + (r.packed ? 4 : 5)) / 2;
+    r.row = 8 * ENTRY_BYTES * (size_t)r.rnx;
     r.slice = r.row * r.rny;
     r.magic = 8388608.0f + (dtype == DT_I16 ? 32768.0f : 0.0f);
     return r;

@@ -28,16 +28,17 @@ struct VolView {
     int pnx, pny, pnz;
 };
 
-// The render layout of a resident volume: each voxel in several entries, so that a sample reads
-// its 64 taps with few aligned wide loads. Entry (x', y', z') holds the 2^3 voxels from (x'-2,
-// y'-2, z'-2), x' in [0, nx+2] and so on, indices clamped to the volume (clamp-to-edge) when
-// the layout is written. A sample at base i reads the 8 entries (i0+1 + {0, 2}, i1+1 + {0, 2},
-// i2+1 + {0, 2}). The voxels lie in pairs along z, one pair per (x, y) with x fastest, as the
-// packed float32 arithmetic of the resampling takes them.
+// The render layout of a resident volume: each voxel in several entries of 16 bytes, so that a
+// sample reads its 64 taps with few aligned wide loads. The entry (x', y', z') starts at voxel
+// (x'-2, y'-2, z'-2), x' in [0, nx+2] and so on, indices clamped to the volume (clamp-to-edge)
+// when the layout is written. The voxels lie in pairs along z with x fastest, as the packed
+// float32 arithmetic of the resampling takes them.
 //
-// 16-bit: 16 bytes, a pair one word (low half the lower z), each voxel plus `bias` as an
-//   unsigned 16-bit value.
-// float32: 32 bytes.
+// 16-bit: the 2^3 voxels, a pair one word (low half the lower z), each voxel plus `bias` as an
+//   unsigned 16-bit value. A sample at base i reads the 8 entries (i0+1 + {0, 2}, i1+1 + {0, 2},
+//   i2+1 + {0, 2}).
+// float32: the 2^2 voxels along x and z (y' in [0, ny+3]); a sample reads 16 entries, i1+1 + {0,
+//   1, 2, 3} along y.
 //
 // Entries lie in blocks of 2^3 (slot 4 (z' & 1) + 2 (y' & 1) + (x' & 1)), blocks in rows along x.
 // The render is bound by the L1 data path, which serves a line at a time: the samples of a warp
@@ -45,8 +46,12 @@ struct VolView {
 // Second phase of a dense 1024^2 frame of a 512^2 x 400 int16 CT, 105 M samples: 2.50 ms and 637
 // M wavefronts of the L1 data path in rows of entries, 2.36 ms and 563 M in blocks, 2.11 ms and
 // 481 M (72% of its rate; 75% of the issue slots) with table lookups of 32 bytes and a kernel per
-// voxel type as well. 256^3 float32 (17 M samples): 0.61 ms and 168 M with 16 loads of four
-// voxels along x in half the memory, 0.53 ms and 125 M so.
+// voxel type as well.
+// float32 entries of 2^3 voxels (8 loads of 32 bytes a sample) would take twice the memory and a
+// third longer to write (256^3: 133 against 99 us). A dense 1280 x 1024 frame of 253 x 187 x 250
+// takes 1.37 ms so and 1.31 ms with them, without bricks 2.77 and 2.40 ms; rays a lane each,
+// whose warps spread over more lines, 2.37 and 2.79 ms (pre-integrated), and a training pass of
+// 256^3 at 512^2 6.29 and 6.45 ms.
 struct ReplView {
     const void *base;
     size_t row, slice;  // bytes from a block to the next along y and z
@@ -171,6 +176,7 @@ __device__ __forceinline__ f32x2 voxels2(uint32_t w, f32x2 sub) {
 
 // Entry (x', y', z') = (x + 2, y + 2, z + 2): the one that starts at voxel (x, y, z). Two entries
 // on along an axis lies the same slot of the next block: 8 entries on along x, 8 rnx along y.
+constexpr int ENTRY_BYTES = 16;
 __device__ __forceinline__ unsigned entry_index(const ReplView &rp, int x, int y, int z) {
     const unsigned X = x + 2, Y = y + 2, Z = z + 2;
     return (((Z >> 1) * rp.rny + (Y >> 1)) * rp.rnx + (X >> 1)) * 8u +
@@ -184,12 +190,17 @@ __device__ __forceinline__ void load32(const void *p, f32x2 v[4]) {
         : "l"(p));
 }
 
-// An entry as it lies in memory.
+// Two pairs of float32 from a 16-byte boundary, through the read-only path.
+__device__ __forceinline__ void load16(const void *p, f32x2 v[2]) {
+    asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "l"(p));
+}
+
+// The 2^3 voxels from (x, y, z) as they lie in memory: one 16-bit entry, or two of float32, the
+// second one voxel on along y (next_y bytes further).
 template <bool PACKED>
 struct Entry {
-    static constexpr size_t SIZE = 16;
     uint4 w;
-    __device__ __forceinline__ void load(const char *p) { w = __ldg((const uint4 *)p); }
+    __device__ __forceinline__ void load(const char *p, int) { w = __ldg((const uint4 *)p); }
     // pair (x, y) = (k & 1, k >> 1) as float32
     __device__ __forceinline__ f32x2 pair(int k, f32x2 sub) const {
         return voxels2(k == 0 ? w.x : k == 1 ? w.y : k == 2 ? w.z : w.w, sub);
@@ -197,24 +208,33 @@ struct Entry {
 };
 template <>
 struct Entry<false> {
-    static constexpr size_t SIZE = 32;
     f32x2 v[4];
-    __device__ __forceinline__ void load(const char *p) { load32(p, v); }
+    __device__ __forceinline__ void load(const char *p, int next_y) {
+        load16(p, v);
+        load16(p + next_y, v + 2);
+    }
     __device__ __forceinline__ f32x2 pair(int k, f32x2) const { return v[k]; }
 };
 
-// The first of a sample's 8 entries, and entry (x, y, z) of them.
-template <bool PACKED>
-__device__ __forceinline__ const char *first_entry(const ReplView &rp, const int ip[3]) {
-    return (const char *)rp.base +
-           Entry<PACKED>::SIZE * (size_t)entry_index(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+// Bytes from an entry at voxel y to the next along y: two slots on in the block, or the same slots
+// of the next block (blocks begin at even y).
+__device__ __forceinline__ int next_entry_y(const ReplView &rp, int y) {
+    return (y & 1) ? (int)rp.row - 2 * ENTRY_BYTES : 2 * ENTRY_BYTES;
 }
-template <bool PACKED>
+
+// The entry at voxel (x, y, z); the first of the 2^3 sets of 2^3 voxels of a sample, and set (x,
+// y, z) of them.
+__device__ __forceinline__ const char *entry_ptr(const ReplView &rp, int x, int y, int z) {
+    return (const char *)rp.base + ENTRY_BYTES * (size_t)entry_index(rp, x, y, z);
+}
+__device__ __forceinline__ const char *first_entry(const ReplView &rp, const int ip[3]) {
+    return entry_ptr(rp, ip[0] - 1, ip[1] - 1, ip[2] - 1);
+}
 __device__ __forceinline__ const char *entry_at(const ReplView &rp, const char *p, int x, int y,
                                                 int z) {
     if (z) p += rp.slice;
     if (y) p += rp.row;
-    return x ? p + 8 * Entry<PACKED>::SIZE : p;
+    return x ? p + 8 * ENTRY_BYTES : p;
 }
 
 // Calls fn(c, b, v) for the 16 tap rows (y ip1-1+b, z ip2-1+c) of base ip, c outermost; v holds
@@ -222,15 +242,16 @@ __device__ __forceinline__ const char *entry_at(const ReplView &rp, const char *
 template <bool PACKED, class Fn>
 __device__ __forceinline__ void for_rows_of(const ReplView &rp, const int ip[3], Fn fn) {
     const f32x2 sub = pack2(-rp.magic, -rp.magic);
-    const char *p = first_entry<PACKED>(rp, ip);
+    const char *p = first_entry(rp, ip);
+    const int ny = next_entry_y(rp, ip[1] - 1);
 #pragma unroll
     for (int zh = 0; zh < 2; ++zh) {
         float4 v[2][4];  // rows of the lower and the upper z
 #pragma unroll
         for (int yh = 0; yh < 2; ++yh) {
             Entry<PACKED> l, u;
-            l.load(entry_at<PACKED>(rp, p, 0, yh, zh));
-            u.load(entry_at<PACKED>(rp, p, 1, yh, zh));
+            l.load(entry_at(rp, p, 0, yh, zh), ny);
+            u.load(entry_at(rp, p, 1, yh, zh), ny);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const float2 a = unpack2(l.pair(2 * k, sub)), b = unpack2(l.pair(2 * k + 1, sub));
@@ -257,12 +278,17 @@ template <bool PACKED>
 __device__ __forceinline__ float tricubic_of(const ReplView &rp, const int ip[3],
                                              const float f[3]) {
     const f32x2 sub = pack2(-rp.magic, -rp.magic);
-    const char *p = first_entry<PACKED>(rp, ip);
+    const char *p = first_entry(rp, ip);
+    const int ny = next_entry_y(rp, ip[1] - 1);
+    // 16-bit: all loads in flight together; float32 takes twice the registers: z half by z half
+    // (with checkpoints 904 -> 776 us for a 640 x 512 image of 253 x 187 x 250 without bricks)
     Entry<PACKED> e[2][2][2];
+    auto load = [&](int zh) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k)
-        e[k >> 2][(k >> 1) & 1][k & 1].load(
-            entry_at<PACKED>(rp, p, k & 1, (k >> 1) & 1, k >> 2));
+        for (int k = 0; k < 4; ++k)
+            e[zh][k >> 1][k & 1].load(entry_at(rp, p, k & 1, k >> 1, zh), ny);
+    };
+    if (PACKED) load(0), load(1);
     float wx[4], wy[4], wz[4];
     bspline_w(f[0], wx);
     bspline_w(f[1], wy);
@@ -277,6 +303,7 @@ __device__ __forceinline__ float tricubic_of(const ReplView &rp, const int ip[3]
 #pragma unroll
     for (int zh = 0; zh < 2; ++zh) {
         f32x2 plane = 0ull;
+        if (!PACKED) load(zh);
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
             const Entry<PACKED> &l = e[zh][b >> 1][0], &u = e[zh][b >> 1][1];
@@ -328,8 +355,7 @@ template <bool PACKED>
 __device__ __forceinline__ void taps8_of(const ReplView &rp, const int ip[3], float v[8]) {
     const f32x2 sub = pack2(-rp.magic, -rp.magic);
     Entry<PACKED> e;
-    e.load((const char *)rp.base +
-           Entry<PACKED>::SIZE * (size_t)entry_index(rp, ip[0], ip[1], ip[2]));
+    e.load(entry_ptr(rp, ip[0], ip[1], ip[2]), next_entry_y(rp, ip[1]));
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float2 z = unpack2(e.pair(k, sub));
@@ -407,15 +433,16 @@ __device__ __forceinline__ float tricubic_grad_of(const ReplView &rp, const int 
         wx2[k] = pack2(wx[k], wx[k]);
         dx2[k] = pack2(dx[k], dx[k]);
     }
-    const char *p = first_entry<PACKED>(rp, ip);
+    const char *p = first_entry(rp, ip);
+    const int ny = next_entry_y(rp, ip[1] - 1);
 #pragma unroll
     for (int zh = 0; zh < 2; ++zh) {
         f32x2 ps = 0ull, pdx = 0ull, pdy = 0ull;
 #pragma unroll
         for (int yh = 0; yh < 2; ++yh) {
             Entry<PACKED> l, u;
-            l.load(entry_at<PACKED>(rp, p, 0, yh, zh));
-            u.load(entry_at<PACKED>(rp, p, 1, yh, zh));
+            l.load(entry_at(rp, p, 0, yh, zh), ny);
+            u.load(entry_at(rp, p, 1, yh, zh), ny);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
                 const int b = 2 * yh + k;
