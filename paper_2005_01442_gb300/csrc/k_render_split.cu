@@ -31,8 +31,17 @@ __global__ void __launch_bounds__(32 * SPLIT_RAY_WARPS, 16 / SPLIT_RAY_WARPS)
 // loads better than 24 at 80 registers (a 1024^2 frame of a 256^3 CT / with soft tissue: 438 /
 // 1290 us against 448 / 1311, with 16 at 128 registers 533 / 1515, with 40 at 48 registers, which
 // spill, 461 / 1460).
+// Float32 volumes with cubic taps: three, at 80 registers. Their taps take twice the registers of
+// 16-bit ones, and cubic pre-classification spilled 480 bytes at 64. 640 x 512 frame of 253 x 187
+// x 250, four CTAs / three: pre-classified 354 / 315 us (with soft tissue 1673 / 1376), shaded
+// 178 / 179 (514 / 479), default 163 / 160 (396 / 373); at 1280 x 1024 the default takes 455 /
+// 469 (1371 / 1322).
+constexpr int tail_ctas_per_sm(int mode, int packed) {
+    return packed == 0 && mode != MODE_LINEAR_POST && mode != MODE_LINEAR_PRE ? 3 : 4;
+}
 template <bool ESL, int MODE, bool CKPT, int PACKED>
-__global__ void __launch_bounds__(32 * SPLIT_WARPS, 4) split_tail_kernel(RenderLaunch L) {
+__global__ void __launch_bounds__(32 * SPLIT_WARPS, tail_ctas_per_sm(MODE, PACKED))
+    split_tail_kernel(RenderLaunch L) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // The counters of the stream's next render: the render before this one, which used them, has
     // ended, and the next one starts after this one. Whatever they hold, each frame starts clean.
@@ -41,30 +50,26 @@ __global__ void __launch_bounds__(32 * SPLIT_WARPS, 4) split_tail_kernel(RenderL
 }
 
 namespace {
-int tail_ctas(cudaError_t &e) {
+int sm_count(cudaError_t &e) {
     static int cached[64] = {0};
     int dev = 0;
     e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return 0;
     if (dev >= 0 && dev < 64 && cached[dev]) return cached[dev];
-    int sms = 0, per_sm = 0;
+    int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, split_tail_kernel<true, MODE_CUBIC_POST, false, 1>, 32 * SPLIT_WARPS, 0);
-    if (e != cudaSuccess) return 0;
-    const int n = sms * (per_sm > 0 ? per_sm : 1);
-    if (dev >= 0 && dev < 64) cached[dev] = n;
-    return n;
+    if (dev >= 0 && dev < 64) cached[dev] = sms;
+    return sms;
 }
 }  // namespace
 
 template <int MODE, bool CKPT, int PACKED>
-static cudaError_t launch_tail_of(const RenderLaunch &L, int ctas, cudaStream_t st) {
+static cudaError_t launch_tail_of(const RenderLaunch &L, int sms, cudaStream_t st) {
     // launched while the first phase ends (programmatic dependent launch; it waits for that end
     // before it reads anything): a 128^2 preview takes 48.4 us instead of 51.1
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
+    cfg.gridDim = dim3(sms * tail_ctas_per_sm(MODE, PACKED));
     cfg.blockDim = dim3(32 * SPLIT_WARPS);
     cfg.stream = st;
     cudaLaunchAttribute attr = {};
@@ -76,14 +81,14 @@ static cudaError_t launch_tail_of(const RenderLaunch &L, int ctas, cudaStream_t 
                   : cudaLaunchKernelEx(&cfg, split_tail_kernel<false, MODE, CKPT, PACKED>, L);
 }
 template <int MODE, bool CKPT = false>
-static cudaError_t launch_tail(const RenderLaunch &L, int ctas, cudaStream_t st) {
-    return L.rep.packed ? launch_tail_of<MODE, CKPT, 1>(L, ctas, st)
-                        : launch_tail_of<MODE, CKPT, 0>(L, ctas, st);
+static cudaError_t launch_tail(const RenderLaunch &L, int sms, cudaStream_t st) {
+    return L.rep.packed ? launch_tail_of<MODE, CKPT, 1>(L, sms, st)
+                        : launch_tail_of<MODE, CKPT, 0>(L, sms, st);
 }
 
 cudaError_t launch_render_split(const RenderLaunch &L, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
-    const int ctas = tail_ctas(e);
+    const int sms = sm_count(e);
     if (e != cudaSuccess) return e;
     const long tiles = (long)((L.cam.width + 7) / 8) * ((L.cam.height + 3) / 4);
     const unsigned grid = (unsigned)((tiles + SPLIT_RAY_WARPS - 1) / SPLIT_RAY_WARPS);
@@ -97,13 +102,13 @@ cudaError_t launch_render_split(const RenderLaunch &L, cudaStream_t st) {
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    if (ck) return launch_tail<MODE_CUBIC_POST, true>(L, ctas, st);
+    if (ck) return launch_tail<MODE_CUBIC_POST, true>(L, sms, st);
     switch (L.mode) {
-    case MODE_LINEAR_POST: return launch_tail<MODE_LINEAR_POST>(L, ctas, st);
-    case MODE_CUBIC_PRE: return launch_tail<MODE_CUBIC_PRE>(L, ctas, st);
-    case MODE_LINEAR_PRE: return launch_tail<MODE_LINEAR_PRE>(L, ctas, st);
-    case MODE_CUBIC_PHONG: return launch_tail<MODE_CUBIC_PHONG>(L, ctas, st);
-    default: return launch_tail<MODE_CUBIC_POST>(L, ctas, st);
+    case MODE_LINEAR_POST: return launch_tail<MODE_LINEAR_POST>(L, sms, st);
+    case MODE_CUBIC_PRE: return launch_tail<MODE_CUBIC_PRE>(L, sms, st);
+    case MODE_LINEAR_PRE: return launch_tail<MODE_LINEAR_PRE>(L, sms, st);
+    case MODE_CUBIC_PHONG: return launch_tail<MODE_CUBIC_PHONG>(L, sms, st);
+    default: return launch_tail<MODE_CUBIC_POST>(L, sms, st);
     }
 }
 

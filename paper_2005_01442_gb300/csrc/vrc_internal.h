@@ -49,7 +49,7 @@ struct VolView {
 // voxel type as well.
 // float32 entries of 2^3 voxels (8 loads of 32 bytes a sample) would take twice the memory and a
 // third longer to write (256^3: 133 against 99 us). A dense 1280 x 1024 frame of 253 x 187 x 250
-// takes 1.37 ms so and 1.31 ms with them, without bricks 2.77 and 2.40 ms; rays a lane each,
+// takes 1.32 ms so and 1.31 ms with them, without bricks 2.75 and 2.40 ms; rays a lane each,
 // whose warps spread over more lines, 2.37 and 2.79 ms (pre-integrated), and a training pass of
 // 256^3 at 512^2 6.29 and 6.45 ms.
 struct ReplView {
