@@ -34,7 +34,9 @@
 // of their taps, so a box of 16 gives some 4.9 atomic sectors a sample instead. 256^3 float32 at
 // 512^2, soft tissue visible (17 M samples): 1.80 ms a view against 4.0 ms. What bounds it now is
 // the chain of a warp's adds and the registers (16 warps an SM): 54% of the issue slots, 61% of
-// the L1 and shared-memory data path.
+// the L1 and shared-memory data path. Eight warps a CTA share the long rays of a tile out better
+// than four and halve the sums that go to the table: 256^3 at 512^2, bone and vessels visible, 298
+// us against 398; with soft tissue 2.06 ms against 2.12.
 #include "vrc_internal.h"
 
 namespace vrc {
@@ -67,11 +69,11 @@ __device__ __forceinline__ void add_taps_x(float *row, int x0, int nx, float v0,
     atomicAdd(row + min(max(x0 + 3, 0), nx - 1), v3);
 }
 
-constexpr int ADJ_WARPS = 4;
+constexpr int ADJ_WARPS = 8;
 constexpr int ADJ_BOX = 1152;    // floats of a warp's box of voxel gradients
 constexpr int ADJ_CHUNK = 16;    // samples summed into one box
 constexpr int ADJ_REC = 36;      // words of a sample's record (conflict-free 16-byte stores)
-constexpr int ADJ_TILE = 32;     // pixels of a CTA at most
+constexpr int ADJ_TILE = 64;     // pixels of a CTA at most
 
 // A ray of the CTA's tile that composited something.
 struct AdjRay {
@@ -88,12 +90,18 @@ struct alignas(16) AdjWarp {  // a warp's shared memory
     float rec[(ADJ_CHUNK + 1) * ADJ_REC];
 };
 
+struct AdjShared {  // a CTA's (dynamic: above the 48 KB of static shared memory)
+    AdjWarp warp[ADJ_WARPS];
+    AdjRay ray[ADJ_TILE];
+};
+
 // NB: blocks of 32 samples that a segment spans at most.
 template <bool ESL, bool VOLGRAD, int NB>
-__global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunch A, int tw_shift,
+__global__ void __launch_bounds__(32 * ADJ_WARPS, 2) adjoint_kernel(AdjointLaunch A, int tw_shift,
                                                                     int th_shift) {
-    __shared__ AdjWarp s_warp[ADJ_WARPS];
-    __shared__ AdjRay s_ray[ADJ_TILE];
+    extern __shared__ AdjShared s_adj[];
+    AdjWarp *const s_warp = s_adj->warp;
+    AdjRay *const s_ray = s_adj->ray;
     __shared__ int s_count, s_head;
     const RenderLaunch &L = A.L;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -391,27 +399,33 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS, 4) adjoint_kernel(AdjointLaunc
 }
 
 template <int NB>
-static void launch_adjoint_n(const AdjointLaunch &A, cudaStream_t st) {
-    // a tile of 8 x 4 pixels a CTA, or 4 x 4 where 8 x 4 would leave SMs without one; not fewer:
-    // every CTA adds its table sums to the same 1024 floats, whose error grows with the number of
-    // additions (4 x 2: 1.5 times the error of 4 x 4 for a 98 x 460 image)
+static cudaError_t launch_adjoint_n(const AdjointLaunch &A, cudaStream_t st) {
+    // Every CTA adds its table sums to the same 1024 floats, whose error grows with the number of
+    // additions (4 x 2 pixels a CTA: 1.5 times the error of 4 x 4 for a 98 x 460 image), so larger
+    // images take larger tiles: 64 pixels from 1.5 Mi on (error of the table gradient of 256^3 at
+    // 2048^2 / 4096^2, random loss: 1.2e-6 / 2.8e-6, with 32 pixels 2.0e-6 / 5.4e-6), 32 from 64 Ki
+    // on, 16 below. Small images want small tiles anyway, large ones large: 256^3 at 128^2 79 us
+    // with 16 pixels, 106 with 32; at 256^2 126, 144 and 208 with 64; at 1024^2 893, 806, 888; at
+    // 1448^2 1740, 1491, 1504 (table alone 1272, 1033, 932); at 2048^2 3650, 3031, 2750.
     const long pixels = (long)A.L.cam.width * A.L.cam.height;
-    const int tw = pixels < 64 * 1024 ? 2 : 3, th = 2;
+    const int tw = pixels < 1536 * 1024 ? 2 : 3, th = pixels < 64 * 1024 ? 2 : 3;
     const unsigned grid = (unsigned)((((long)A.L.cam.width + (1 << tw) - 1) >> tw) *
                                      ((A.L.cam.height + (1 << th) - 1) >> th));
     const bool esl = A.L.dist != nullptr, vg = A.grad_vol != nullptr;
-    if (esl && vg) adjoint_kernel<true, true, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
-    else if (esl) adjoint_kernel<true, false, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
-    else if (vg) adjoint_kernel<false, true, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
-    else adjoint_kernel<false, false, NB><<<grid, 32 * ADJ_WARPS, 0, st>>>(A, tw, th);
+    auto kernel = esl ? (vg ? adjoint_kernel<true, true, NB> : adjoint_kernel<true, false, NB>)
+                      : (vg ? adjoint_kernel<false, true, NB> : adjoint_kernel<false, false, NB>);
+    const cudaError_t e = cudaFuncSetAttribute(
+        kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AdjShared));
+    if (e != cudaSuccess) return e;
+    kernel<<<grid, 32 * ADJ_WARPS, sizeof(AdjShared), st>>>(A, tw, th);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint(const AdjointLaunch &A, cudaStream_t st) {
     static_assert(ADJ_MAX_SEG <= 128, "a segment spans at most 4 blocks of 32 samples");
-    if (A.seg <= 32) launch_adjoint_n<1>(A, st);
-    else if (A.seg <= 64) launch_adjoint_n<2>(A, st);
-    else launch_adjoint_n<4>(A, st);
-    return cudaGetLastError();
+    if (A.seg <= 32) return launch_adjoint_n<1>(A, st);
+    if (A.seg <= 64) return launch_adjoint_n<2>(A, st);
+    return launch_adjoint_n<4>(A, st);
 }
 
 }  // namespace vrc
