@@ -31,8 +31,8 @@ struct Bricks {
 struct Occ {
     uint8_t *dev = nullptr;   // occupancy bytes
     uint8_t *dist = nullptr;  // 8 forward-box distance fields (0 = occupied)
-    uint8_t *fine = nullptr;  // B = 16: the distance fields of 8^3 tiles (build_fine)
-    int *scratch = nullptr;   // used while building the fields (and, B = 16, the tile bytes)
+    uint8_t *fine = nullptr;  // B = 16, TILE_MIN_BRICKS: the distance fields of 8^3 tiles
+    int *scratch = nullptr;   // used while building the fields (and, with tiles, their bytes)
     uint32_t *cells = nullptr;  // cell transparency mask (cellmask_bytes)
     long n = 0;
     unsigned brick_version = 0, tf_version = 0;
@@ -368,7 +368,22 @@ void tile_counts(const Volume &v, int nt[3]) {
 // the cell mask also gives the occupancy of 8^3 tiles, and fields for leaping over them
 // (fine_out): a ray then leaps over seven eighths of a brick that is occupied in one corner.
 // 512^2 x 2000 at 4096^2, quarter-voxel steps: 3.48 -> 2.52 ms a frame; a shaded 777 x 613 frame
-// of 253 x 187 x 250: 298 -> 271 us. The fields of 64 x 64 x 50 tiles take 26 us a rebuild.
+// of 253 x 187 x 250: 298 -> 271 us. The fields of 64 x 64 x 50 tiles take 26 us a rebuild. Volumes
+// of few bricks do without: 64^3, 2% of a 512^2 frame against 15 of 66 us a rebuild.
+constexpr long TILE_MIN_BRICKS = 128;
+
+// Whether a render of `pixels` pixels leaps over the tiles of a volume of `bricks` bricks of 16, or
+// over the bricks: smaller boxes end closer to what is visible, but take more leaps, one after
+// the other. Split and TMA-staged render and groups of 4 and 8 lanes: where an image has enough
+// rays to hide those (CT of 192^3, tiles / bricks: 160 x 120 75 / 68 us, 256^2 91 / 87, 512 x 384
+// 127 / 131; 512^2 x 400 at 1024^2 351 / 457). A lane a ray and groups of 32 and 16 lanes march
+// whole warps by their longest ray: in large volumes only (kernel 1, 640 x 512: 253 x 187 x 250
+// 403 / 348 us, 400^3 500 / 480, 512^2 x 400 at 1024^2 660 / 675; kernel 2 418 / 389, 613 / 695).
+bool leaps_over_tiles(int kernel, long pixels, long bricks) {
+    if (kernel == 1 || kernel == 2 || kernel == 5) return bricks >= 16384;
+    return pixels >= 64 * 1024;
+}
+
 vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStream_t st,
                       const uint8_t **out, const uint8_t **dist_out = nullptr,
                       const uint32_t **cells_out = nullptr, const uint8_t **fine_out = nullptr) {
@@ -393,7 +408,7 @@ vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStre
         o.n = 0;
         CK(cudaMalloc(&o.dev, (size_t)b.count()), "cudaMalloc(occupancy)");
         CK(cudaMalloc(&o.dist, 8 * (size_t)b.count()), "cudaMalloc(occupancy)");
-        if (B == 16) {
+        if (B == 16 && b.count() >= TILE_MIN_BRICKS) {
             CK(cudaMalloc(&o.fine, 8 * (size_t)nt[0] * nt[1] * nt[2]), "cudaMalloc(occupancy)");
             CK(cudaMalloc(&o.scratch, align256(box_dist_scratch_bytes(nt)) +
                                           (size_t)nt[0] * nt[1] * nt[2]), "cudaMalloc(occupancy)");
@@ -410,7 +425,7 @@ vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStre
         CK(launch_box_dist(o.dev, b.nb, o.scratch, o.dist, st), "distance launch");
         CK(launch_cellmask(view_of(v), B, b.nb, o.dev, t.dev->zrun, t.lo, t.du, o.cells, st),
            "cell mask launch");
-        if (B == 16) {
+        if (o.fine) {
             uint8_t *tiles = (uint8_t *)o.scratch + align256(box_dist_scratch_bytes(nt));
             CK(launch_tile_occupancy(o.cells, v.n, nt, tiles, st), "tile occupancy launch");
             CK(launch_box_dist(tiles, nt, o.scratch, o.fine, st), "distance launch");
@@ -634,7 +649,8 @@ vrc_status prepare_render(vrc_ctx *ctx, int vol_id, int tf_id, const vrc_camera 
         for (int k = 0; k < 3; ++k) L.bricks.nb[k] = b.nb[k];
         L.bricks.mn = b.mn;
         L.bricks.mx = b.mx;
-        if (tiles && fine) {
+        if (tiles && fine &&
+            leaps_over_tiles(p->kernel, (long)cam->width * cam->height, b.count())) {
             L.dist = fine;
             L.bricks.B = 8;
             L.bricks.shift = 3;
