@@ -130,6 +130,8 @@ struct vrc_ctx {
     int *err_word = nullptr;   // device error word shared by kernels
     float4 *host_img = nullptr;  // device image for vrc_render_host
     size_t host_img_bytes = 0;
+    uint32_t *mask_rows = nullptr;  // rows of vrc_cellmask_get, grown to the largest mask
+    size_t mask_rows_bytes = 0;
     std::map<cudaStream_t, SplitBuf> split;  // split-render queues by stream
     std::map<cudaStream_t, CaptureBuf> captured;  // and those of renders captured on a stream
     std::map<int, Plan> plans;               // piece grids (vrc_pieces_build)
@@ -828,6 +830,7 @@ vrc_status vrc_destroy(vrc_ctx *ctx) {
     for (auto &kv : ctx->tfs) free_tf(kv.second);
     cudaFree(ctx->err_word);
     cudaFree(ctx->host_img);
+    cudaFree(ctx->mask_rows);
     for (auto &kv : ctx->split) cudaFree(kv.second.base);
     for (auto &kv : ctx->captured) {
         cudaFree(kv.second.base);
@@ -1092,15 +1095,18 @@ vrc_status vrc_cellmask_get(vrc_ctx *ctx, int vol_id, int tf_id, int B, uint32_t
     const uint32_t *cells = nullptr;
     vrc_status s = ensure_occ(ctx, *v, tf_id, *t, B, st, &occ, nullptr, &cells);
     if (s != VRC_OK) return s;
-    uint32_t *rows = nullptr;
-    cudaError_t e = cudaMalloc(&rows, sizeof(uint32_t) * (size_t)nwords);
-    if (e == cudaSuccess) e = launch_cellmask_rows(cells, v->n, rows, st);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(words_host, rows, sizeof(uint32_t) * (size_t)nwords,
-                            cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaFree(rows);
-    CK(e, "cell mask copy");
+    const size_t bytes = sizeof(uint32_t) * (size_t)nwords;
+    if (ctx->mask_rows_bytes < bytes) {  // (no call leaves work on it behind)
+        cudaFree(ctx->mask_rows);
+        ctx->mask_rows = nullptr;
+        ctx->mask_rows_bytes = 0;
+        CK(cudaMalloc(&ctx->mask_rows, bytes), "cudaMalloc(cell mask rows)");
+        ctx->mask_rows_bytes = bytes;
+    }
+    CK(launch_cellmask_rows(cells, v->n, ctx->mask_rows, st), "cell mask rows launch");
+    CK(cudaMemcpyAsync(words_host, ctx->mask_rows, bytes, cudaMemcpyDeviceToHost, st),
+       "cell mask copy");
+    CK(cudaStreamSynchronize(st), "cell mask copy sync");
     return VRC_OK;
 }
 
