@@ -334,9 +334,9 @@ vrc_status vrc_server_destroy(vrc_server *s);
  * the cell transparency mask is rebuilt there too when it fits behind the brick fields,
  * else samples in transparent cells are resampled (same pixels, more executed samples).
  * params->kernel 6 (split render) is rejected with VRC_ERR_ARG: its queue needs memory.
- * Returns VRC_ERR_ARG, with a message naming the sizes, when the brick grid needs more than
- * the array holds (about 9 bytes per brick plus a 4-byte summed-volume table entry per
- * brick). All calls share the one array: calls that can overlap on the GPU (other streams,
+ * Returns VRC_ERR_ARG, with a message naming the sizes, when the brick grid is too large for
+ * the array, counted as 9 bytes per brick plus 4 per corner of the grid, (nbx+1)(nby+1)(nbz+1)
+ * of them. All calls share the one array: calls that can overlap on the GPU (other streams,
  * other contexts of the process) race and must be serialised by the caller.
  * The paper has no counterpart to this call. */
 vrc_status vrc_render_noalloc(vrc_ctx *ctx, int vol_id, int tf_id, const vrc_camera *cam,

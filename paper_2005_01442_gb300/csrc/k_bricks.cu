@@ -838,16 +838,14 @@ __global__ void __launch_bounds__(256) dist_axis4_kernel(const uint32_t *__restr
     }
 }
 
-size_t box_dist_scratch_bytes(const int nb[3]) {
-    return (size_t)(nb[0] + 1) * (nb[1] + 1) * (nb[2] + 1) * sizeof(int);
-}
+size_t box_dist_scratch_bytes(const int nb[3]) { return 4 * (size_t)nb[0] * nb[1] * nb[2]; }
 
 // The x fields go through the first quarter of `dist`, the y fields (4 bytes a brick) through
 // `scratch`.
-cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], int *scratch, uint8_t *dist,
+cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], uint8_t *scratch, uint8_t *dist,
                              cudaStream_t st) {
     const long n = (long)nb[0] * nb[1] * nb[2], rows = (long)nb[1] * nb[2];
-    uint8_t *yf = (uint8_t *)scratch;
+    uint8_t *yf = scratch;
     dist_x_kernel<<<(unsigned)((rows + DX_WARPS - 1) / DX_WARPS), 32 * DX_WARPS, 0, st>>>(
         occ, nb[0], rows, dist);
     auto blocks = [](long k) { return (unsigned)((k + 255) / 256 > 152L * 64 ? 152L * 64

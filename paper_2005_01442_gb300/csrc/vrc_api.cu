@@ -32,7 +32,7 @@ struct Occ {
     uint8_t *dev = nullptr;   // occupancy bytes
     uint8_t *dist = nullptr;  // 8 forward-box distance fields (0 = occupied)
     uint8_t *fine = nullptr;  // B = 16, TILE_MIN_BRICKS: the distance fields of 8^3 tiles
-    int *scratch = nullptr;   // used while building the fields (and, with tiles, their bytes)
+    uint8_t *scratch = nullptr;  // used while building the fields (and, with tiles, their bytes)
     uint32_t *cells = nullptr;  // cell transparency mask (cellmask_bytes)
     long n = 0;
     unsigned brick_version = 0, tf_version = 0;
@@ -428,7 +428,7 @@ vrc_status ensure_occ(vrc_ctx *ctx, Volume &v, int tf_id, Tf &t, int B, cudaStre
         CK(launch_cellmask(view_of(v), B, b.nb, o.dev, t.dev->zrun, t.lo, t.du, o.cells, st),
            "cell mask launch");
         if (o.fine) {
-            uint8_t *tiles = (uint8_t *)o.scratch + align256(box_dist_scratch_bytes(nt));
+            uint8_t *tiles = o.scratch + align256(box_dist_scratch_bytes(nt));
             CK(launch_tile_occupancy(o.cells, v.n, nt, tiles, st), "tile occupancy launch");
             CK(launch_box_dist(tiles, nt, o.scratch, o.fine, st), "distance launch");
         }
@@ -1429,16 +1429,19 @@ extern "C" vrc_status vrc_render_noalloc(vrc_ctx *ctx, int vol_id, int tf_id,
     Tf *t = get_tf(ctx, tf_id);
     if (!t) return fail(ctx, VRC_ERR_ARG, "unknown transfer function id %d", tf_id);
     Bricks *b = nullptr;
-    size_t occ_off = 0, dist_off = 0, svt_off = 0, cells_off = 0;
+    size_t occ_off = 0, dist_off = 0, fields_off = 0, cells_off = 0;
     if (B) {
         b = &v->bricks[slot_of(B)];
         if (!b->mn || b->B != B) return fail(ctx, VRC_ERR_STATE, "brick table B=%d not built", B);
         const size_t n = (size_t)b->count();
         occ_off = 0;
         dist_off = align256(n);
-        svt_off = dist_off + align256(8 * n);
-        const size_t need = svt_off + align256(box_dist_scratch_bytes(b->nb));
-        cells_off = need;
+        fields_off = dist_off + align256(8 * n);
+        cells_off = fields_off + align256(box_dist_scratch_bytes(b->nb));
+        // the documented limit: 4 bytes per corner of the grid, although the fields need them per
+        // brick only
+        const size_t need = fields_off + align256(4 * (size_t)(b->nb[0] + 1) * (b->nb[1] + 1) *
+                                                  (b->nb[2] + 1));
         if (need > (size_t)VRC_NOALLOC_SCRATCH_BYTES)
             return fail(ctx, VRC_ERR_ARG,
                         "vrc_render_noalloc: %ld bricks of size %d need %zu scratch bytes, above "
@@ -1457,11 +1460,10 @@ extern "C" vrc_status vrc_render_noalloc(vrc_ctx *ctx, int vol_id, int tf_id,
         if (s != VRC_OK) return s;
         uint8_t *occ = scratch + occ_off;
         uint8_t *dist = scratch + dist_off;
-        int *svt = (int *)(scratch + svt_off);
         // every byte these kernels read is written first by this call: nothing to clear
         CK(launch_occupancy(b->mn, b->mx, v->dtype, b->count(), t->dev->prefix, t->lo, t->du, occ, st),
            "occupancy launch");
-        CK(launch_box_dist(occ, b->nb, svt, dist, st), "distance launch");
+        CK(launch_box_dist(occ, b->nb, scratch + fields_off, dist, st), "distance launch");
         // the cell mask too when it fits behind the tables (it only saves work)
         if (cells_off + cellmask_bytes(v->n) <= (size_t)VRC_NOALLOC_SCRATCH_BYTES) {
             uint32_t *cells = (uint32_t *)(scratch + cells_off);
@@ -1996,7 +1998,8 @@ vrc_status vrc_pieces_build(vrc_ctx *ctx, int vol_id, int tf_id, int B, const in
 
     // device work: per piece the masked occupancy and its distance fields, then the boxes
     uint8_t *mask = nullptr;
-    int *scratch = nullptr, *dk = nullptr;
+    uint8_t *scratch = nullptr;
+    int *dk = nullptr;
     std::vector<int> boxes((size_t)6 * K);
     cudaError_t e = cudaMalloc(&mask, (size_t)b.count());
     if (e == cudaSuccess) e = cudaMalloc(&scratch, box_dist_scratch_bytes(b.nb));

@@ -750,7 +750,7 @@ cudaError_t launch_cellmask_rows(const uint32_t *cells, const int n[3], uint32_t
                                  cudaStream_t st);
 size_t box_dist_scratch_bytes(const int nb[3]);
 // dist: 8 x nbricks bytes (one forward-box distance field per direction octant)
-cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], int *scratch, uint8_t *dist,
+cudaError_t launch_box_dist(const uint8_t *occ, const int nb[3], uint8_t *scratch, uint8_t *dist,
                              cudaStream_t st);
 // Object-order pieces and sort-last compositing (k_pieces.cu).
 constexpr int MAX_PIECES = 64;
