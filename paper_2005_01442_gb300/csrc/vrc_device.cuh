@@ -362,8 +362,9 @@ __device__ __forceinline__ void bspline_dw(float f, float w[4]) {
 
 constexpr float ALPHA_MAX = 0.99999994039535522f;  // 1 - 2^-24
 
-// The logarithm and exponential units as they are, flushing denormals: without the scaling that
-// __log2f and exp2f put around them for arguments and results below 2^-126.
+// The PTX approximations of the logarithm and the exponential to base 2, which flush subnormal
+// operands and results to zero. Their documented errors: lg2 2^-22 (absolute in (0.5, 2), else
+// relative), ex2 2^-22 (relative).
 __device__ __forceinline__ float lg2(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -375,8 +376,8 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
-// Opacity of a segment of length delta for table opacity a per unit length. (1 - a is no denormal,
-// and a power below 2^-126 leaves 1 - 0 = 1 as any would: the same bits as with __log2f, exp2f.)
+// Opacity of a segment of length delta for table opacity a per unit length. 1 - a >= 2^-24 is not
+// subnormal, and a power that is flushed to zero is far below the rounding of the 1 - it goes to.
 __device__ __forceinline__ float segment_alpha(float a, float delta) {
     a = fminf(fmaxf(a, 0.0f), ALPHA_MAX);
     return 1.0f - ex2(delta * lg2(1.0f - a));
