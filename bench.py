@@ -240,6 +240,23 @@ def measure_peaks(R, sms: int) -> dict:
                       f"{sms} SMs"}
 
 
+def rebuild_launches(brick: int, dims) -> int:
+    """Kernels of a brick table and its occupancy: bricks, occupancy, 3 distance passes, cell mask;
+    with bricks of 16 (128 or more of them) also the 8^3 tiles and their 3 distance passes."""
+    bricks = math.prod(-(-n // brick) for n in dims)
+    return 10 if brick == 16 and bricks >= 128 else 6
+
+
+def counted_by(brick: int) -> str:
+    """What the executed samples of a workload are. Counting renders leap over the bricks
+    asked for; with bricks of 16 the timed ones leap over 8^3 tiles, so there executed samples
+    are those of occupied 16^3 bricks whether or not the timed kernel visits them."""
+    if brick == 16:
+        return ("samples in occupied 16^3 bricks; the timed renders leap over 8^3 tiles and visit "
+                "fewer (resampled samples do not depend on it)")
+    return f"samples in occupied {brick}^3 bricks" if brick else "all samples up to termination"
+
+
 def roofline(executed: int, resampled: int, launch_ms: float, peaks: dict, kernel: str) -> dict:
     """Roofline of one render call: max(N F / P_fp32, N G / BW_L1) over its CUDA-event time,
     N = executed samples (`frac`) or resampled samples (`frac_resampled`)."""
@@ -505,15 +522,15 @@ def main():
             "mrays_per_s": world * rays_per_step * args.steps / secs / 1e6,
             "gsamples_nominal_per_s": world * nominal * args.steps / secs / 1e9,
             "samples_per_step": {"nominal": nominal, "executed": executed,
-                                 "resampled": resampled},
+                                 "resampled": resampled, "executed_are": counted_by(B)},
             "render_kernel_ms": kernel_ms,
             "roofline": roof,
             "fp32_sgemm_tflops_measured": sgemm,
             "other_workloads_and_kernels": legs,
             "cpu_baseline": cpu, "e2e": e2e,
-            # bricks, occupancy, 3 distance passes, cell mask; per frame the
-            # split render's two kernels (one for the per-ray kernel)
-            "gpu_launches": args.steps * (6 + args.cameras * (2 if args.kernel in (0, 6) else 1)),
+            # the rebuild; per frame the split render's two kernels (one for the other kernels)
+            "gpu_launches": args.steps * (rebuild_launches(B, dims) +
+                                          args.cameras * (2 if args.kernel in (0, 6) else 1)),
             "clocks": clocks,
         }
         if not args.no_serve:
@@ -793,7 +810,9 @@ def run_mode(args, torch, R, synth):
             "mode": "variants", "metric": "ms per frame; PSNR / SSIM vs tricubic "
             "post-classification (RGBA, peak 1)", "data": "synthetic",
             "config": workload_config(args), "variants": rows,
-            "gpu_launches": 7 * (args.warmup + args.steps) * len(cams) * 2, "clocks": _clocks()}), flush=True)
+            # two kernels a split render, one for the pre-integrated variant
+            "gpu_launches": (2 * (len(rows) - 1) + 1) * args.steps * len(cams),
+            "clocks": _clocks()}), flush=True)
         return
     if args.mode == "sortlast":
         # object-order rendering: the headline workload cut into grids of pieces of whole
@@ -931,7 +950,10 @@ def run_mode(args, torch, R, synth):
             "nominal_samples": nominal, "executed_samples": executed,
             "resampled_samples": resampled, "checkpoint_bytes": int(ck.numel()),
             "render_ms": p_ms, "forward_with_checkpoints_ms": f_ms, "backward_ms": b_ms,
+            "executed_are": counted_by(B),
             "forward_gsamples_per_s": executed / (p_ms / 1e3) / 1e9,
+            "forward_gsamples_resampled_per_s": resampled / (p_ms / 1e3) / 1e9,
+            "forward_gsamples_nominal_per_s": nominal / (p_ms / 1e3) / 1e9,
             "mrays_per_s": 4096 * 4096 / (p_ms / 1e3) / 1e6, "clocks": _clocks()}), flush=True)
         return
 

@@ -213,7 +213,9 @@ vrc_status vrc_cellmask_get(vrc_ctx *ctx, int vol_id, int tf_id, int B, uint32_t
  * nominal samples (segments inside the box, summed over rays), executed samples (samples
  * up to termination that lie in occupied bricks, or every sample up to termination when
  * params->brick = 0; those in clear cells are counted though not resampled) and resampled
- * samples (the executed ones that were resampled and composited).
+ * samples (the executed ones that were resampled and composited). With counters a render leaps
+ * over the bricks asked for; without them, with bricks of 16, it may leap over 8^3 tiles within
+ * them as well (the same image), so executed samples are then not the ones it visits.
  * ckpt_dev: NULL, or a caller-owned device buffer of vrc_ckpt_bytes(cam, params, vol_id, ctx)
  * bytes (256-byte aligned) that the render fills with the checkpoints vrc_render_backward
  * needs (see there): the ray of every pixel records its first checkpointed segment and its
