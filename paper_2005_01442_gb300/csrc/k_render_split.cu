@@ -28,7 +28,7 @@ __global__ void __launch_bounds__(32 * SPLIT_RAY_WARPS, 16 / SPLIT_RAY_WARPS)
 }
 
 // Four CTAs per SM (64 registers, a few spills): 32 resident warps hide the latency of dependent
-// loads better than 24 at 80 registers (a 1024^2 frame of a 256^3 CT / with soft tissue: 438 /
+// loads better than 24 at 80 registers (1024^2 frame of a 256^3 int16 CT / with soft tissue: 438 /
 // 1290 us against 448 / 1311, with 16 at 128 registers 533 / 1515, with 40 at 48 registers, which
 // spill, 461 / 1460).
 // Float32 volumes with cubic taps: three, at 80 registers. Their taps take twice the registers of

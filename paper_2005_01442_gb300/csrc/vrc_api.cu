@@ -871,8 +871,8 @@ vrc_status vrc_volume_upload(vrc_ctx *ctx, const void *data, int on_device, vrc_
     const size_t es = dtype_size(dtype);
     const size_t padded = (size_t)v.pnx * v.pny * v.pnz * es;
     const size_t raw = (size_t)nx * ny * nz * es;
-    if ((size_t)v.pnx * v.pny * v.pnz >= (size_t)1 << 31 ||
-        (size_t)(nx + 1) * (ny + 4) * (nz + 4) >= (size_t)1 << 31)
+    // (the render layout has at most (nx + 5)(ny + 5)(nz + 5) entries, counted in 32 bits)
+    if ((size_t)v.pnx * v.pny * v.pnz >= (size_t)1 << 31)
         return fail(ctx, VRC_ERR_ARG, "volume too large (padded elements must stay below 2^31)");
     cudaError_t e = cudaMalloc(&v.dpad, padded);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMalloc(volume)");
